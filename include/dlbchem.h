@@ -94,15 +94,20 @@ typedef struct dlbchem_options {
   double map_Ytol;      /* absolute composition tolerance (1e-4) */
   double map_Tmax;      /* > 0: only cells below this T qualify (0 = off) */
   int32_t team_warps;   /* warps per cell: 1, 2, 4, or 0 = automatic (1 up to 32 unknowns, 2 up to 64, else 4) */
-  int32_t precision;    /* 0: FP64 LU of the iteration matrix (default); 1: FP32 LU with FP64
-                           iterative refinement: residuals against the FP64 matrix, stopped when
-                           the estimated remaining error is below 1e-6 of the error weights, at
-                           most 3 rounds, the step redone with the FP64 LU if they do not
-                           converge. State, rates, error norm and step control stay FP64.
-                           Fixed at create, which then allocates one FP64 matrix copy per
-                           resident team (SMs x CTAs per SM x teams x N^2 doubles; 22 MB at 54
-                           unknowns on 152 SMs); integrations of such a context always launch
-                           persistent teams (the plain schedule keeps index order). */
+  int32_t precision;    /* 0: linear solves to FP64 accuracy (default): up to 32 unknowns per
+                           warp of the team by an FP32 inverse of the iteration matrix and FP64
+                           iterative refinement (residuals against the FP64 matrix) until the
+                           last correction is below 2^-30 of the solution, at most 8 rounds;
+                           beyond that size, and for a step whose refinement does not converge,
+                           by the FP64 LU. 1: mixed precision: the refinement (beyond the size
+                           above with FP32 LU factors) stops when the estimated remaining error
+                           is below 1e-6 of the error weights, at most 3 rounds, the step redone
+                           with the FP64 LU if they do not converge. State, rates, error norm
+                           and step control are FP64 in both. Fixed at create, which allocates
+                           one matrix per resident team (SMs x CTAs per SM x teams; 22 MB at 54
+                           unknowns on 152 SMs); if that fails, precision 0 runs the FP64 LU
+                           throughout and precision 1 returns OOM. Mixed-precision contexts always
+                           launch persistent teams (the plain schedule keeps index order). */
   int32_t predictor;    /* 1: order the queue by the attached network's predicted step counts
                            (no previous call needed); steps[] is then only written */
   int32_t surrogate;    /* 1: try the attached network's increments first; cells that pass the
@@ -299,7 +304,7 @@ int dlbchem_nreactions(const dlbchem_ctx* ctx);
  *   with mapping 2; see dlbchem_last_mapping), out[3] team size in threads, out[4] teams per CTA,
  *   out[5] CTAs launched by the integrator, out[6] dynamic shared memory
  *   bytes per CTA, out[7] kernel launches in the call, out[8] steps whose
- *   FP32 refinement fell back to the FP64 LU, out[9] precision mode.
+ *   mixed-precision refinement fell back to the FP64 LU, out[9] precision mode.
  * Returns DLBCHEM_OK, BAD_ARG or CUDA.
  */
 int dlbchem_last_stats(dlbchem_ctx* ctx, int64_t out[10]);

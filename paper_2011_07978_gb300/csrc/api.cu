@@ -959,12 +959,22 @@ int dlbchem_create(const char* mech_path, const dlbchem_options* opt, dlbchem_ct
   // so that callers who reserve their memory after creating the context
   // find it in place (a failure here is retried by the first static call)
   (void)dlb::static_scratch_prepare(c->device);
-  if (o.precision == 1) {
-    const size_t slots = size_t(c->num_sms) * c->blocks_per_sm * c->teams;
-    if (cudaMalloc(&c->d_m64, slots * c->dm.N * c->dm.N * sizeof(double)) != cudaSuccess) {
+  if (o.precision == 1 || c->dm.N <= 32 * c->wpc) {
+    const size_t slots = size_t(c->num_sms) * c->blocks_per_sm;
+    const std::vector<unsigned> zero(slots, 0u);
+    if (cudaMalloc(&c->d_m64, slots * c->teams * dlb::matrix_stride(c->dm.N, c->dm.CH) * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&c->d_slots, slots * sizeof(unsigned)) != cudaSuccess ||
+        cudaMemcpy(c->d_slots, zero.data(), slots * sizeof(unsigned), cudaMemcpyHostToDevice) != cudaSuccess) {
+      if (o.precision == 1) {
+        dlbchem_destroy(c);
+        return fail(nullptr, DLBCHEM_OOM, "device allocation of the mixed-precision matrix copies failed");
+      }
+      // no room: this context keeps the FP64 LU, which needs none
+      cudaGetLastError();
+      if (c->d_m64) cudaFree(c->d_m64);
+      if (c->d_slots) cudaFree(c->d_slots);
       c->d_m64 = nullptr;
-      dlbchem_destroy(c);
-      return fail(nullptr, DLBCHEM_OOM, "device allocation of the mixed-precision matrix copies failed");
+      c->d_slots = nullptr;
     }
   }
   *out = c;
@@ -1063,8 +1073,8 @@ int dlbchem_integrate(dlbchem_ctx* c, int64_t n, double dt, const double* T, con
   a.P.max_steps = c->opt.max_steps; a.P.isothermal = c->opt.isothermal; a.P.precision = c->opt.precision;
   a.L = c->L;
   a.n = n; a.T = T; a.p = p; a.Y = Y; a.Tout = T_out; a.Yout = Y_out; a.steps = steps; a.status = status;
-  a.fallbacks = c->d_counter + 2;
-  a.m64 = c->opt.precision == 1 ? c->d_m64 : nullptr;
+  a.fallbacks = c->opt.precision == 1 ? c->d_counter + 2 : nullptr;   // counted for mixed precision only
+  c->matrix_slots(a);
   if (c->opt.precision == 1 && (e = cudaMemsetAsync(c->d_counter + 2, 0, 8, s)) != cudaSuccess)
     return cuda_fail(c, e, "cudaMemsetAsync");
   const bool listed = mapping || queue || surrogate || predictor;
@@ -1364,6 +1374,7 @@ void dlbchem_destroy(dlbchem_ctx* c) {
   if (c->d_counter) cudaFree(c->d_counter);
   if (c->d_ws) cudaFree(c->d_ws);
   if (c->d_m64) cudaFree(c->d_m64);
+  if (c->d_slots) cudaFree(c->d_slots);
   if (c->d_learn) cudaFree(c->d_learn);
   for (auto& ev : c->ev)
     if (ev) cudaEventDestroy(ev);

@@ -118,7 +118,8 @@ struct IntegParams {
 // Offsets (in doubles) of one team's workspace inside dynamic shared memory.
 struct WsLayout {
   int M, y0, f0, ys, fs, u, c, E, Einv, hk, wdot, vv, dwdT, uu, invd, q, dqdT, dlt, D, scal, perm;
-  int M32, invd32, perm32, rr, dx, isc;   // mixed precision only (else 0-sized)
+  int M32, invd32, perm32, rr, dx, isc;   // mixed precision with more unknowns than threads only (else 0)
+  int w32, v, keys, rows;                 // refined solves with the FP32 inverse
   int total;  // doubles per team (int and float arrays are counted in doubles)
 };
 
@@ -148,7 +149,22 @@ __host__ inline WsLayout make_layout(int nsp, int nrx, int CH, int N, int ld, in
   L.scal = take(48);
   L.perm = take((N + 1) / 2 + 1);
   L.M32 = L.invd32 = L.perm32 = L.rr = L.dx = L.isc = 0;
-  if (mixed) {
+  // refined solves: weights and right-hand side over the Jacobian-only arrays
+  // dwdT .. dlt (dead from the assembly of one step to the next), keys and
+  // published rows (dead during the rate evaluations too) behind them up to scal
+  L.w32 = L.v = L.keys = L.rows = 0;
+  if (N <= CH) {
+    const int warps = CH / 32;
+    auto vectors = [&](auto&& take2) {
+      L.w32 = take2((N + 1) / 2);
+      L.v = take2(CH / 2);
+      L.keys = take2(warps);
+      L.rows = take2(warps * CH);
+    };
+    int o2 = L.dwdT;
+    vectors([&](int n) { int r = o2; o2 += (n + 1) & ~1; return r; });
+    if (o2 > L.scal) vectors(take);
+  } else if (mixed) {
     // FP32 factors over the first half of M (the FP64 matrix is kept in a
     // global per-team scratch); pivots and refinement vectors over the
     // Jacobian-only arrays dwdT .. dlt, dead from the factorisation to the
@@ -172,6 +188,13 @@ __host__ inline WsLayout make_layout(int nsp, int nrx, int CH, int N, int ld, in
   }
   L.total = o;
   return L;
+}
+
+// Doubles of one team's matrix in the global scratch: M (mixed precision) or the
+// FP32 inverse, N rows of at most CH floats; 16-byte aligned.
+__host__ __device__ inline int64_t matrix_stride(int N, int CH) {
+  const int64_t a = int64_t(N) * N, b = (int64_t(N) * CH + 1) / 2;
+  return ((a > b ? a : b) + 1) & ~int64_t(1);
 }
 
 // One mesh of a batched launch: its arrays, size and flow step.
@@ -211,9 +234,11 @@ struct KernelArgs {
   int chunk;
   int queue;
   unsigned long long* fallbacks;   // steps whose FP32 refinement fell back to the FP64 LU
-  // mixed precision: per-team FP64 matrices (N*N doubles each, transposed),
-  // indexed by blockIdx.x * teams + team; launches are then persistent
+  // refined solves: per-team matrices (matrix_stride doubles each): a CTA takes
+  // slot i of nslots (slots[i] 0 -> 1) for its teams while it runs
   double* m64;
+  unsigned* slots;
+  int nslots, slots_per_sm;
   // batched launch (nmesh > 0): work-list entries are (mesh << kMeshShift) | cell
   // and each mesh brings its own arrays and dt; the single-mesh fields above
   // are then unused.

@@ -52,7 +52,16 @@ struct dlbchem_ctx {
   // workspace (grown on demand to the largest ncells seen)
   unsigned long long* d_counter = nullptr;   // queue counter (8 B) + reference index (8 B)
   void* d_ws = nullptr;
-  double* d_m64 = nullptr;   // mixed precision: per-team FP64 matrix copies (resident teams x N^2)
+  // refined solves: matrices (resident teams x matrix_stride doubles) and the flags of
+  // their slots (one per resident CTA)
+  double* d_m64 = nullptr;
+  unsigned* d_slots = nullptr;
+  void matrix_slots(dlb::KernelArgs& a) const {
+    a.m64 = d_m64;
+    a.slots = d_slots;
+    a.nslots = d_m64 ? num_sms * blocks_per_sm : 0;
+    a.slots_per_sm = blocks_per_sm;
+  }
   int64_t ws_cap = 0;
   uint8_t* w_flag = nullptr;
   double* w_ref_state = nullptr;

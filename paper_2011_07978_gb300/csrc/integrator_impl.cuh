@@ -20,6 +20,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "dlb_common.cuh"
 
@@ -124,6 +125,14 @@ struct Team {
   }
 };
 
+// Scratch of the refined solves (invert and solve_inverse below).
+struct InvScratch {
+  int* pinv;        // [N] column whose pivot row i was
+  float* rows;      // [2][WPC][NP] published rows
+  unsigned* keys;   // [2][WPC]
+  float* v;         // [NP] right-hand side in pivot order
+};
+
 struct WS {
   double *M, *y0, *f0, *ys, *fs, *u, *c, *E, *Einv, *hk, *wdot, *vv, *dwdT, *uu, *invd, *q, *dqdT, *dlt,
       *D, *scal;
@@ -131,9 +140,12 @@ struct WS {
   float *M32, *invd32;
   int* perm32;
   double *rr, *dx, *isc;
+  InvScratch inv;         // refined solves with the FP32 inverse
+  float* inv_isc;
   const double* exptab;   // 64 entries of 2^(j/64), shared by the CTA
   const double* nutab;    // nutab[j] = j - 8: stoichiometric coefficients by their 4-bit code
-  double* g;              // mixed precision: this team's FP64 matrix, transposed (global, L2-resident)
+  double* g;              // this team's global scratch (L2-resident): the FP32 inverse, or mixed
+                          // precision's FP64 matrix, transposed
 };
 
 __device__ __forceinline__ WS carve(double* base, const WsLayout& L) {
@@ -146,6 +158,9 @@ __device__ __forceinline__ WS carve(double* base, const WsLayout& L) {
   w.M32 = reinterpret_cast<float*>(base + L.M32); w.invd32 = reinterpret_cast<float*>(base + L.invd32);
   w.perm32 = reinterpret_cast<int*>(base + L.perm32);
   w.rr = base + L.rr; w.dx = base + L.dx; w.isc = base + L.isc;
+  w.inv = InvScratch{w.perm, reinterpret_cast<float*>(base + L.rows), reinterpret_cast<unsigned*>(base + L.keys),
+                     reinterpret_cast<float*>(base + L.v)};
+  w.inv_isc = reinterpret_cast<float*>(base + L.w32);
   return w;
 }
 
@@ -163,8 +178,9 @@ struct Mix {
 // 2^m is added to the exponent field. tab[j] = 2^(j/64) rounded to double.
 // About 10 FP64 operations against ~19 for the library exp; |x| >= 700 and
 // NaN go to the library exp.
+static __device__ __noinline__ double exp_library(double x) { return exp(x); }   // one copy, off the hot path
 __device__ __forceinline__ double exp_tab(double x, const double* __restrict__ tab) {
-  if ((__double2hiint(x) & 0x7fffffff) >= 0x4085E000) return exp(x);   // |x| >= 700 or NaN (700 = 0x4085E000 00000000)
+  if ((__double2hiint(x) & 0x7fffffff) >= 0x4085E000) return exp_library(x);   // |x| >= 700 or NaN (700 = 0x4085E000 00000000)
   const double kShift = 6755399441055744.0;                 // 1.5 * 2^52
   const double t = fma(x, 92.33248261689366, kShift);       // x * 64 / ln2, rounded to an integer
   const int ki = __double2loint(t);
@@ -475,6 +491,7 @@ __device__ __forceinline__ void eval_rates(const DevMech& m, const Team<WPC>& tm
     }
     tm.sync();
     double* qa = w.D;
+#pragma unroll 1
     for (int r = tm.tid; r < nrx; r += TS) reaction<false, GEN>(m, w, mx, r, r, qa);
     tm.sync();
     for (int rd = m.incp_all[tm.warp], r1 = m.incp_all[tm.warp + 1]; rd < r1; ++rd) {
@@ -998,6 +1015,216 @@ __device__ __forceinline__ float trunc_to_float(double v) {
   return __uint_as_float(sign | f);
 }
 
+// double -> float by truncating the significand (integer operations: the FP64
+// unit does conversions at its own rate). Magnitudes below the float normal
+// range flush to zero; above it, infinity and NaN become infinite or NaN.
+__device__ __forceinline__ float low_float(double v) {
+  const unsigned hi = unsigned(__double2hiint(v)), t = hi & 0x7fffffffu;
+  unsigned f = __funnelshift_l(unsigned(__double2loint(v)), t - 0x38000000u, 3);
+  f = t < 0x38100000u ? 0u : (t >= 0x47f00000u ? 0x7f800000u : f);
+  return __uint_as_float(f | (hi & 0x80000000u));
+}
+
+// ---------------------------------------------------------------------------
+// Refined solves (a thread per row: N <= NP <= 32 WPC). The FP64 unit is what
+// a step is bound by (one warp instruction per 76 cycles and SM
+// sub-partition, measured, against one per cycle on the FP32 pipe), and with
+// two cells' worth of warps per sub-partition so is the latency of serial
+// code. So M is not factorised in FP64: an FP32 inverse X of M serves as the
+// preconditioner of an FP64 iterative refinement, x <- x + X (b - M x), with
+// the residual against the FP64 matrix. An inverse and not an LU because a
+// triangular sweep is a chain of N columns (8.4 kcycles for 54 unknowns, 12
+// sweeps per step) and a product with X is none.
+// Measured per step, FP64 LU and solves before: 53 species, two warps per
+// cell, 224 -> 149 us alone on an SM, 309 -> 241 us with six cells (FP64 warp
+// instructions 5,040 -> about 3,300); 100 species, four warps, 540 -> 332 us
+// with two cells; 10 species, one warp, 51 -> 43 us. The error against a
+// 64-bit integration is the same (1.3e-14 and 1.4e-14 relative in Y on 4,001
+// cells of 53 species, 1.1e-13 and 1.1e-13 on 400 of 100).
+//
+// Gauss-Jordan elimination in registers: thread i holds row i. Per column each
+// warp's best pivot row publishes itself (key and row, double-buffered), one
+// barrier, and every thread subtracts its multiple of the best of those rows.
+// Columns rotate: element j moves to j - 1 as it is updated, the pivot column
+// is always element 0 and the new column of the inverse enters at the end, so
+// that every register index is fixed in a loop over the columns. A pivot row is
+// scaled once, at the end. Rows stay where they are: the row that was pivot
+// of column m ends as row m of X with the columns in pivot order, so X is
+// applied to a right-hand side in that order (pinv[i] = m). The pivot is a
+// largest |M_ik| to within 2^-16 relative: the 32-bit key is |M_ik| with its 7
+// low bits replaced by 127 - i, so ties go to the lower row. X goes to a
+// global per-team scratch (L2), four columns per 16 bytes: X4[q N + m]. Returns
+// false if a pivot is zero (or below the key's resolution).
+// ---------------------------------------------------------------------------
+template <int WPC, int NP>
+__device__ __noinline__ bool invert(const Team<WPC> tm, const double* M, int N, int ld, const InvScratch sc, float4* X4) {
+  const int row = tm.tid;
+  const bool has = row < N;
+  bool live = has;
+  int m = 0;
+  float scale = 0.f;
+  float a[NP];
+  const double* src = M + min(row, N - 1) * ld;
+#pragma unroll
+  for (int j = 0; j < NP; ++j) a[j] = has && j < N ? low_float(src[j]) : 0.f;
+  volatile unsigned* keys = sc.keys;
+  for (int k = 0; k < N; ++k) {
+    const unsigned key = live ? (__float_as_uint(a[0]) & 0x7fffff80u) | unsigned(127 - row) : 0u;
+    const unsigned best = __reduce_max_sync(0xffffffffu, key);
+    const int buf = (k & 1) * WPC;
+    if ((best >> 7) == 0u) {
+      if (tm.lane == 0) keys[buf + tm.warp] = 0u;
+    } else if (key == best) {
+      keys[buf + tm.warp] = best;
+      float4* dst = reinterpret_cast<float4*>(sc.rows + (buf + tm.warp) * NP);
+#pragma unroll
+      for (int q = 0; q < NP / 4; ++q) dst[q] = make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
+    }
+    tm.sync();
+    unsigned top = keys[buf];
+    int from = buf;
+#pragma unroll
+    for (int w = 1; w < WPC; ++w) {
+      const unsigned kw = keys[buf + w];
+      if (kw > top) { top = kw; from = buf + w; }
+    }
+    if (top == 0u) return false;   // the same in every thread
+    const float4* u4 = reinterpret_cast<const float4*>(sc.rows + from * NP);
+    float4 u = u4[0];
+    float rp;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rp) : "f"(u.x));
+    const bool piv = has && row == 127 - int(top & 127u);
+    const float nf = piv ? 0.f : -(a[0] * rp);
+    if (piv) {
+      live = false;
+      m = k;
+      scale = rp;
+    }
+    a[0] = fmaf(nf, u.y, a[1]);
+    a[1] = fmaf(nf, u.z, a[2]);
+    a[2] = fmaf(nf, u.w, a[3]);
+#pragma unroll
+    for (int q = 1; q < NP / 4; ++q) {
+      u = u4[q];
+      a[4 * q - 1] = fmaf(nf, u.x, a[4 * q]);
+      a[4 * q] = fmaf(nf, u.y, a[4 * q + 1]);
+      a[4 * q + 1] = fmaf(nf, u.z, a[4 * q + 2]);
+      a[4 * q + 2] = fmaf(nf, u.w, a[4 * q + 3]);
+    }
+    a[NP - 1] = piv ? 1.f : nf;
+  }
+  for (int k = N; k < NP; ++k) {   // the unused columns go round to the end
+    const float t = a[0];
+#pragma unroll
+    for (int j = 0; j + 1 < NP; ++j) a[j] = a[j + 1];
+    a[NP - 1] = t;
+  }
+  if (has) {
+    sc.pinv[row] = m;
+#pragma unroll
+    for (int q = 0; q < NP / 4; ++q)
+      __stcg(X4 + q * N + m, make_float4(a[4 * q] * scale, a[4 * q + 1] * scale, a[4 * q + 2] * scale, a[4 * q + 3] * scale));
+  }
+  tm.sync();
+  return true;
+}
+
+// x = M^-1 b by the refinement above. With the error weights isc = 1/sc, dmax
+// = max |d_i| isc_i of the last correction d and xmax = max |x_i| isc_i:
+//  - tight (the default, FP64 accuracy): done when dmax <= 2^-30 xmax. The
+//    correction's own relative error is that of a product with X, 2^-24 cond,
+//    so what is left is below 2^-54 cond, the error of an FP64 LU. Two
+//    rounds reach it unless 2^-24 cond > 2^-15; at most eight are tried.
+//  - mixed precision (the caller's choice): done when the error left, dmax
+//    rho / (1 - rho), is below 1e-6, with rho estimated by dmax / xmax after
+//    the first correction and by the ratio of successive corrections after
+//    that; at most three rounds.
+// Returns false if it did not converge (the caller then takes the FP64 LU).
+template <int WPC, int NP>
+__device__ __noinline__ bool solve_inverse(const Team<WPC> tm, const double* M, int N, int ld, const InvScratch sc,
+                                           const float4* X4, const double* b, double* x, const float* isc, bool tight) {
+  const int t = tm.tid;
+  const bool has = t < N;
+  const int i = min(t, N - 1);
+  float4 xr[NP / 4];   // row i of X, for every round
+#pragma unroll
+  for (int q = 0; q < NP / 4; ++q) xr[q] = __ldcg(X4 + q * N + i);
+  const int at = sc.pinv[i];
+  const double bi = b[i];
+  const float wi = isc[i];
+  const double* row = M + i * ld;
+  auto apply = [&]() {
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    const float4* v4 = reinterpret_cast<const float4*>(sc.v);
+#pragma unroll
+    for (int q = 0; q < NP / 4; ++q) {
+      const float4 v = v4[q];
+      s0 = fmaf(xr[q].x, v.x, s0);
+      s1 = fmaf(xr[q].y, v.y, s1);
+      s2 = fmaf(xr[q].z, v.z, s2);
+      s3 = fmaf(xr[q].w, v.w, s3);
+    }
+    return (s0 + s1) + (s2 + s3);
+  };
+  if (has) sc.v[at] = low_float(bi);
+  else if (t < NP) sc.v[t] = 0.f;
+  tm.sync();
+  double xi = double(apply());
+  if (has) x[i] = xi;
+  tm.sync();
+  float prev = 0.f;
+  for (int it = 0; it < (tight ? 8 : 3); ++it) {
+    double r0 = bi, r1 = 0.0;
+    int j = 0;
+#pragma unroll 4
+    for (; j + 1 < N; j += 2) {
+      r0 = fma(-row[j], x[j], r0);
+      r1 = fma(-row[j + 1], x[j + 1], r1);
+    }
+    if (j < N) r0 = fma(-row[j], x[j], r0);
+    if (has) sc.v[at] = low_float(r0 + r1);
+    tm.sync();
+    const float d = apply();
+    xi += double(d);
+    if (has) x[i] = xi;
+    if (tight && it == 0) { tm.sync(); continue; }
+    // maxima of values that are non-negative, infinite or NaN, by bit pattern
+    unsigned ud = has ? __float_as_uint(fabsf(d) * wi) : 0u;
+    unsigned ux = has ? __float_as_uint(fabsf(low_float(xi)) * wi) : 0u;
+    tm.umax2(ud, ux);
+    if (WPC == 1) __syncwarp();
+    const float hd = __uint_as_float(ud), hx = __uint_as_float(ux);
+    if (!(hd < 1e38f) || !(hx < 1e38f)) return false;
+    if (tight) {
+      if (hd <= 9.3132257e-10f * hx) return true;
+    } else {
+      if (hd == 0.f) return true;
+      const float rho = it == 0 ? hd / hx : hd / prev;
+      if (rho < 1.f && hd * rho <= 1e-6f * (1.f - rho)) return true;
+    }
+    prev = hd;
+  }
+  return false;
+}
+
+// The padded sizes that are compiled: a multiple of four, at most 32 WPC.
+template <int WPC, class F>
+__device__ __forceinline__ auto with_padded(int N, F&& f) {
+  if constexpr (WPC == 1) {
+    if (N <= 12) return f(std::integral_constant<int, 12>());
+    if (N <= 20) return f(std::integral_constant<int, 20>());
+    return f(std::integral_constant<int, 32>());
+  } else if constexpr (WPC == 2) {
+    if (N <= 40) return f(std::integral_constant<int, 40>());
+    if (N <= 56) return f(std::integral_constant<int, 56>());
+    return f(std::integral_constant<int, 64>());
+  } else {
+    if (N <= 80) return f(std::integral_constant<int, 80>());
+    if (N <= 104) return f(std::integral_constant<int, 104>());
+    return f(std::integral_constant<int, 128>());
+  }
+}
+
 // Walk the N x N elements e = t, t + TS, ... as (i, j) = (e % N, e / N)
 // with incremental indices (no division per element).
 template <int TS, class F>
@@ -1022,7 +1249,7 @@ __device__ __forceinline__ double wrms(const Team<WPC>& tm, const double* v, con
 // Starting step (Hairer, Norsett, Wanner, Solving ODEs I, Sec. II.4) with the
 // order-3 error exponent 1/4 and fallbacks scaled by dt. Uses ys, fs, u.
 template <int WPC, bool GEN>
-__device__ double initial_step(const DevMech& m, const Team<WPC>& tm, const WS& w, const IntegParams& P,
+__device__ __forceinline__ double initial_step(const DevMech& m, const Team<WPC>& tm, const WS& w, const IntegParams& P,
                                double P1, double iP1, bool iso) {
   constexpr int TS = 32 * WPC;
   const int N = m.N;
@@ -1047,7 +1274,7 @@ __device__ double initial_step(const DevMech& m, const Team<WPC>& tm, const WS& 
 
 // Integrate one cell over [0, dt] (the oracle's algorithm step for step).
 template <int WPC, bool GEN>
-__device__ void integrate_cell(const DevMech& m, const IntegParams& P, const Team<WPC>& tm, const WS& w,
+__device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegParams& P, const Team<WPC>& tm, const WS& w,
                                int64_t cell, int64_t n, const double* __restrict__ Tin,
                                const double* __restrict__ pin, const double* __restrict__ Yin,
                                double* __restrict__ Tout, double* __restrict__ Yout, int32_t* __restrict__ steps_out,
@@ -1084,9 +1311,21 @@ __device__ void integrate_cell(const DevMech& m, const IntegParams& P, const Tea
       ++steps;
       const double ih = rcp_nr(h);
       assemble<WPC, GEN>(m, tm, w, P1, iP1, iso, ih * (1.0 / kGamma));
-      bool mixed = P.precision == 1 && w.g != nullptr;   // no scratch: FP64
+      // Refined solves with an FP32 inverse where there is a thread per row (the
+      // automatic team sizes up to 128 unknowns); the FP64 matrix stays in
+      // shared memory. Beyond that the FP64 LU, or for mixed precision the FP32
+      // LU. Without scratch always the FP64 LU.
+      bool inverse = w.g != nullptr && N <= TS;
+      bool mixed = w.g != nullptr && P.precision == 1 && !inverse;
       bool ok;
       const int ld = m.ld;
+      float4* X4 = reinterpret_cast<float4*>(w.g);
+      if (inverse) {
+        if (tm.tid < N)
+          w.inv_isc[tm.tid] = __frcp_rn(fmaf(float(P.rtol), fabsf(low_float(w.y0[tm.tid])), fmaxf(float(P.atol), 1e-30f)));
+        ok = with_padded<WPC>(N, [&](auto np) { return invert<WPC, decltype(np)::value>(tm, w.M, N, ld, w.inv, X4); });
+        if (!ok) inverse = false;
+      }
       // mixed: M goes, transposed, to the team's global copy, and its FP32
       // truncation over M's first half is factorised in shared memory;
       // restore() brings the FP64 matrix back for the FP64 fallback
@@ -1107,39 +1346,45 @@ __device__ void integrate_cell(const DevMech& m, const IntegParams& P, const Tea
         else ok = lu_factor<WPC, float>(tm, w.M32, N, ld, w.invd32, w.perm32);
         if (!ok) { mixed = false; restore(); }
       }
-      if (!mixed) ok = lu_factor<WPC, double>(tm, w.M, N, ld, w.invd, w.perm);
+      if (!mixed && !inverse) ok = lu_factor<WPC, double>(tm, w.M, N, ld, w.invd, w.perm);
       for (int attempt = 0; attempt < 2; ++attempt) {
         bool conv = true;
         auto solve = [&](const double* b, double* x) {
-          if (mixed) conv &= solve_refined<WPC>(tm, w.g, w.M32, N, ld, w.invd32, w.perm32, b, x, w.rr, w.dx, w.isc);
+          if (inverse) {
+            conv &= with_padded<WPC>(N, [&](auto np) {
+              return solve_inverse<WPC, decltype(np)::value>(tm, w.M, N, ld, w.inv, X4, b, x, w.inv_isc,
+                                                             P.precision == 0);
+            });
+          } else if (mixed) conv &= solve_refined<WPC>(tm, w.g, w.M32, N, ld, w.invd32, w.perm32, b, x, w.rr, w.dx, w.isc);
           else lu_solve<WPC, double>(tm, w.M, N, m.ld, w.invd, w.perm, b, x);
         };
-        // stage 1
-        solve(w.f0, u1);
-        // stage 2
-        for (int i = tm.tid; i < N; i += TS) w.ys[i] = fma(kA21, u1[i], w.y0[i]);
-        tm.sync();
-        eval_f<WPC, GEN>(m, tm, w, w.ys, P1, iP1, iso, w.fs);
-        for (int i = tm.tid; i < N; i += TS) w.fs[i] = fma(kC21 * ih, u1[i], w.fs[i]);
-        tm.sync();
-        solve(w.fs, u2);
-        // stage 3
-        for (int i = tm.tid; i < N; i += TS) w.ys[i] = fma(kA31, u1[i], fma(kA32, u2[i], w.y0[i]));
-        tm.sync();
-        eval_f<WPC, GEN>(m, tm, w, w.ys, P1, iP1, iso, w.fs);
-        for (int i = tm.tid; i < N; i += TS) w.ys[i] = fma(ih, fma(kC31, u1[i], kC32 * u2[i]), w.fs[i]);
-        tm.sync();
-        solve(w.ys, u3);
-        // stage 4 (same f as stage 3)
-        for (int i = tm.tid; i < N; i += TS)
-          w.ys[i] = fma(ih, fma(kC41, u1[i], fma(kC42, u2[i], kC43 * u3[i])), w.fs[i]);
-        tm.sync();
-        solve(w.ys, u4);
-        if (!mixed || conv) break;
+        // one call site of the solve and of the rate evaluation for all stages
+        // (four inlined copies overflow the instruction cache and the inliner)
+#pragma unroll 1
+        for (int stage = 1; stage <= 4; ++stage) {
+          if (stage == 2 || stage == 3) {   // stage 4 has the f of stage 3
+            for (int i = tm.tid; i < N; i += TS)
+              w.ys[i] = stage == 2 ? fma(kA21, u1[i], w.y0[i]) : fma(kA31, u1[i], fma(kA32, u2[i], w.y0[i]));
+            tm.sync();
+            eval_f<WPC, GEN>(m, tm, w, w.ys, P1, iP1, iso, w.fs);
+          }
+          if (stage > 1) {
+            for (int i = tm.tid; i < N; i += TS) {
+              double v;
+              if (stage == 2) v = fma(kC21 * ih, u1[i], w.fs[i]);
+              else if (stage == 3) v = fma(ih, fma(kC31, u1[i], kC32 * u2[i]), w.fs[i]);
+              else v = fma(ih, fma(kC41, u1[i], fma(kC42, u2[i], kC43 * u3[i])), w.fs[i]);
+              w.ys[i] = v;
+            }
+            tm.sync();
+          }
+          solve(stage == 1 ? w.f0 : w.ys, w.u + (stage - 1) * N);
+        }
+        if (!(mixed || inverse) || conv) break;
         // refinement did not converge: redo the stages with the FP64 LU of the kept matrix
-        mixed = false;
         if (tm.tid == 0 && fallbacks) atomicAdd(fallbacks, 1ull);
-        restore();
+        if (mixed) restore();
+        mixed = inverse = false;
         ok = lu_factor<WPC, double>(tm, w.M, N, ld, w.invd, w.perm);
       }
       // new state (ys) and error estimate
@@ -1200,12 +1445,27 @@ __global__ void __launch_bounds__(128, WPC == 1 ? 4 : (WPC == 2 ? 3 : 2)) rosenb
   double* tab = smem + size_t(teams) * a.L.total;
   for (int j = threadIdx.x; j < 64; j += blockDim.x) tab[j] = a.m.exptab[j];
   for (int j = threadIdx.x; j < 16; j += blockDim.x) tab[64 + j] = double(j - 8);
+  // The CTA takes a free matrix slot for as long as it runs. There are as many
+  // slots as CTAs of this kernel can be resident, so calls that overlap on
+  // the GPU (several streams) find one too; with none free the FP64 LU runs.
+  __shared__ int cta_slot;
+  if (threadIdx.x == 0) {
+    cta_slot = -1;
+    unsigned smid;
+    asm("mov.u32 %0, %%smid;" : "=r"(smid));
+    for (int t = 0; t < a.nslots; ++t) {
+      const int i = int((smid * unsigned(a.slots_per_sm) + unsigned(t)) % unsigned(a.nslots));
+      if (atomicCAS(a.slots + i, 0u, 1u) == 0u) { cta_slot = i; break; }
+    }
+    __threadfence();
+  }
   __syncthreads();
+  const int slot = cta_slot;
   double* base = smem + size_t(team) * a.L.total;
   WS w = carve(base, a.L);
   w.exptab = tab;
   w.nutab = tab + 64;
-  w.g = a.m64 ? a.m64 + (size_t(blockIdx.x) * teams + team) * size_t(a.m.N) * a.m.N : nullptr;
+  w.g = slot >= 0 ? a.m64 + (size_t(slot) * teams + team) * matrix_stride(a.m.N, a.m.CH) : nullptr;
   tm.red = w.scal;
   const int64_t nq = a.nqueue ? *a.nqueue : a.n;
   // one work-list entry -> (arrays, cell, dt)
@@ -1227,7 +1487,7 @@ __global__ void __launch_bounds__(128, WPC == 1 ? 4 : (WPC == 2 ? 3 : 2)) rosenb
   // One call site of run() for both schedules: a second inlined copy of the
   // integrator may contract a*b + c into FMAs differently, and plain and
   // queued runs are meant to give bit-identical results.
-  volatile int64_t* slot = reinterpret_cast<volatile int64_t*>(w.scal + 24);
+  volatile int64_t* pulled = reinterpret_cast<volatile int64_t*>(w.scal + 24);
   bool once = !a.queue;
   for (;;) {
     int64_t first, last;
@@ -1235,9 +1495,9 @@ __global__ void __launch_bounds__(128, WPC == 1 ? 4 : (WPC == 2 ? 3 : 2)) rosenb
       first = int64_t(blockIdx.x) * teams + team;
       last = first + 1;
     } else {
-      if (tm.tid == 0) *slot = int64_t(atomicAdd(a.counter, (unsigned long long)a.chunk));
+      if (tm.tid == 0) *pulled = int64_t(atomicAdd(a.counter, (unsigned long long)a.chunk));
       tm.sync();
-      first = *slot;
+      first = *pulled;
       tm.sync();
       last = first + int64_t(a.chunk);
     }
@@ -1246,7 +1506,13 @@ __global__ void __launch_bounds__(128, WPC == 1 ? 4 : (WPC == 2 ? 3 : 2)) rosenb
     for (int64_t qi = first; qi < last; ++qi) run(a.perm ? int64_t(a.perm[qi]) : qi);
     if (once) break;
   }
+  __syncthreads();
+  if (threadIdx.x == 0 && slot >= 0) {
+    __threadfence();
+    atomicExch(a.slots + slot, 0u);
+  }
 }
+
 
 // ---------------------------------------------------------------------------
 // Surrogate gate: a predicted state (T', Y') = (T, Y) + (dT, dY) (with

@@ -124,7 +124,7 @@ extern "C" int dlbchem_integrate_static(dlbchem_ctx* c, int64_t n, double dt, co
   a.L = c->L;
   a.n = n; a.T = T; a.p = p; a.Y = Y; a.Tout = T_out; a.Yout = Y_out; a.steps = steps; a.status = status;
   a.perm = list; a.nqueue = total; a.queue = 1; a.counter = counter; a.chunk = c->opt.chunk;
-  a.m64 = c->opt.precision == 1 ? c->d_m64 : nullptr;   // allocated once, at creation
+  c->matrix_slots(a);   // allocated once, at creation
   // mixed precision: count the steps whose refinement fell back to the FP64
   // LU in the context's own counter (allocated at creation)
   if (c->opt.precision == 1) {
