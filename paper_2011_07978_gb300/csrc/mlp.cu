@@ -53,19 +53,18 @@ __device__ __forceinline__ float dsilu_f(float z) {
   return s * fmaf(z, 1.0f - s, 1.0f);
 }
 
-// C[M x N] = op(A)[M x K] op(B)[K x N] (+ bias[n]); optional pre-activation
-// copy Z and SiLU. A: TA ? A[k*lda + m] : A[m*lda + k]; B: TB ? B[n*ldb + k]
-// : B[k*ldb + n]. On the fifth-generation tensor cores: BF16 operands (FP32
-// rounded while staged) in shared memory in the canonical K-major layout
-// without swizzle (8 x 8 core matrices of 128 B, the K-groups of a row group
-// contiguous), FP32 accumulator in tensor memory. One CTA of 128 threads
-// computes a 128 x 64 tile: every thread stages, one thread issues the MMAs of
-// a k-tile (K = 16 each) and commits them to an mbarrier, all wait (bounded),
-// then each warp reads its 32 accumulator rows from tensor memory for the
-// epilogue. A wait that gives up sets *status, writes NaN and still frees the
-// tensor memory.
+// C[M x N] = A[M x K] B[K x N] with an epilogue, on the fifth-generation tensor
+// cores: BF16 operands (FP32 rounded while staged) in shared memory in the
+// canonical K-major layout without swizzle (8 x 8 core matrices of 128 B, the
+// K-groups of a row group contiguous), FP32 accumulator in tensor memory. One
+// CTA of 256 threads computes a tile: every thread stages, one thread issues
+// the MMAs of a k-tile (K = 16 each) and commits them to its buffer's mbarrier
+// (two buffers; a buffer is refilled when its MMAs are done, every wait is
+// bounded), then each warp reads 32 accumulator rows from tensor memory for
+// the epilogue. A wait that gives up sets *status, writes NaN and still frees
+// the tensor memory.
 constexpr int kTM = 128, kTN = 64, kTK = 64;
-constexpr uint32_t kTmemCols = 64;
+constexpr int kGemmThreads = 256;
 constexpr int kWaitLimit = 1 << 24;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
@@ -78,110 +77,277 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint3
          (uint64_t((sbo >> 4) & 0x3FFF) << 32) | (uint64_t(1) << 46);
 }
 
-// byte offset of (row, k) in a tile of rows x kTK BF16 values
-__device__ __forceinline__ int tile_off(int row, int k) {
-  return ((row >> 3) * (kTK / 8) + (k >> 3)) * 128 + (row & 7) * 16 + (k & 7) * 2;
+// Staging moves eight values of one row per thread and step: global loads of
+// whole 32-byte sectors (or coalesced over rows), one conflict-free 16-byte
+// store, and the loads of the next two k-tiles are in flight while the tensor
+// cores work on this one. An operand's values of consecutive k are adjacent (KC: p[row ld + k])
+// or those of consecutive rows (p[k ld + row]).
+template <bool KC>
+struct TileSource {
+  const float* p;
+  int ld, rows, kend;   // rows and k beyond these are zero
+  bool vec;             // KC: rows start on 16 bytes
+  __device__ TileSource(const float* p_, int ld_, int rows_, int kend_)
+      : p(p_), ld(ld_), rows(rows_), kend(kend_), vec((ld_ & 3) == 0 && (reinterpret_cast<uintptr_t>(p_) & 15) == 0) {}
+  // chunk e of a tile of ROWS rows: its row and first k
+  template <int ROWS>
+  static __device__ __forceinline__ void place(int e, int& row, int& k) {
+    if (KC) { row = (e & 7) + ((e >> 6) << 3); k = ((e >> 3) & 7) * 8; }
+    else { row = e % ROWS; k = (e / ROWS) * 8; }
+  }
+  __device__ __forceinline__ void load(int row, int k, float* v) const {
+    if (KC) {
+      const float* q = p + int64_t(row) * ld + k;
+      if (vec && row < rows && k + 8 <= kend) {
+        *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(q);
+        *reinterpret_cast<float4*>(v + 4) = *reinterpret_cast<const float4*>(q + 4);
+        return;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = row < rows && k + j < kend ? q[j] : 0.0f;
+    } else {
+      const float* q = p + int64_t(k) * ld + row;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = row < rows && k + j < kend ? q[int64_t(j) * ld] : 0.0f;
+    }
+  }
+};
+
+__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);   // a in the low half (lower k)
+  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <bool TA, bool TB>
-__global__ void __launch_bounds__(128) gemm_tc_kernel(int M, int N, int K, const float* __restrict__ A, int lda,
-                                                      const float* __restrict__ B, int ldb, float* __restrict__ C,
-                                                      int ldc, const float* __restrict__ bias, float* __restrict__ Z,
-                                                      int act, int* __restrict__ status) {
-  __shared__ __align__(1024) unsigned char sop[(kTM + kTN) * kTK * 2];
-  __shared__ __align__(8) unsigned long long mbar;
+// The 128 x NT tile at (m0, n0): epi(gm, gn, v, nv) takes nv <= 16 consecutive
+// columns of one row. With BSUM, bsum[n] (NT floats of shared memory) receives
+// the sums over k of B's FP32 values.
+template <int NT, bool BSUM, bool AKC, bool BKC, class Epi>
+__device__ __forceinline__ void gemm_tile(const TileSource<AKC>& A, const TileSource<BKC>& B, int m0, int n0, float* bsum,
+                                          int* __restrict__ status, Epi&& epi) {
+  constexpr int kNA = kTM * kTK / 8 / kGemmThreads, kNB = NT * kTK / 8 / kGemmThreads;   // chunks per thread
+  constexpr int kBuf = (kTM + NT) * kTK * 2;
+  static_assert(!BSUM || (!BKC && kNB == 1 && NT == 32), "one chunk of one row per thread");
+  __shared__ __align__(1024) unsigned char sop[2 * kBuf];
+  __shared__ __align__(8) unsigned long long mbar[2];
   __shared__ uint32_t tmem_slot;
-  unsigned char* sA = sop;
-  unsigned char* sB = sop + kTM * kTK * 2;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.y * kTM, n0 = blockIdx.x * kTN;
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)) : "memory");
+    for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[b])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
-                 "r"(kTmemCols) : "memory");
+                 "r"(uint32_t(NT)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  float ra[2][kNA][8], rb[2][kNB][8];
+  auto fetch = [&](int set, int k0) {
+    int row, k;
+#pragma unroll
+    for (int i = 0; i < kNA; ++i) {
+      TileSource<AKC>::template place<kTM>(tid + kGemmThreads * i, row, k);
+      A.load(m0 + row, k0 + k, ra[set][i]);
+    }
+#pragma unroll
+    for (int i = 0; i < kNB; ++i) {
+      TileSource<BKC>::template place<NT>(tid + kGemmThreads * i, row, k);
+      B.load(n0 + row, k0 + k, rb[set][i]);
+    }
+  };
+  const int K = A.kend, ntiles = (K + kTK - 1) / kTK;
+  fetch(0, 0);
+  if (ntiles > 1) fetch(1, kTK);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
   // kind::f16 instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, N and M
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(kTN >> 3) << 17) | (uint32_t(kTM >> 4) << 24);
-  uint32_t phase = 0;
-  bool ok = true;
-  for (int k0 = 0; k0 < K && ok; k0 += kTK) {
-    // stage the k-tile (zero outside the matrices)
-    for (int e = tid; e < kTM * kTK; e += 128) {
-      int mm, kk;
-      if (TA) { kk = e / kTM; mm = e % kTM; } else { mm = e / kTK; kk = e % kTK; }
-      const int gm = m0 + mm, gk = k0 + kk;
-      float v = 0.0f;
-      if (gm < M && gk < K) v = TA ? A[int64_t(gk) * lda + gm] : A[int64_t(gm) * lda + gk];
-      *reinterpret_cast<__nv_bfloat16*>(sA + tile_off(mm, kk)) = __float2bfloat16_rn(v);
-    }
-    for (int e = tid; e < kTN * kTK; e += 128) {
-      int nn, kk;
-      if (TB) { nn = e / kTK; kk = e % kTK; } else { kk = e / kTN; nn = e % kTN; }
-      const int gn = n0 + nn, gk = k0 + kk;
-      float v = 0.0f;
-      if (gn < N && gk < K) v = TB ? B[int64_t(gn) * ldb + gk] : B[int64_t(gk) * ldb + gn];
-      *reinterpret_cast<__nv_bfloat16*>(sB + tile_off(nn, kk)) = __float2bfloat16_rn(v);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor cores
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (tid == 0) {
-#pragma unroll
-      for (int kk = 0; kk < kTK / 16; ++kk) {
-        const uint64_t ad = umma_desc(smem_u32(sA) + kk * 256, 128, (kTK / 8) * 128);
-        const uint64_t bd = umma_desc(smem_u32(sB) + kk * 256, 128, (kTK / 8) * 128);
-        const uint32_t acc = (k0 > 0 || kk > 0) ? 1u : 0u;
-        asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-                     "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&mbar))
-                   : "memory");
-    }
-    // every thread waits for this k-tile's MMAs before the tile is overwritten (bounded)
+  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(NT >> 3) << 17) | (uint32_t(kTM >> 4) << 24);
+  auto store = [&](unsigned char* base, int row, int k, const float* v) {
+    *reinterpret_cast<uint4*>(base + ((row >> 3) * (kTK / 8) + (k >> 3)) * 128 + (row & 7) * 16) =
+        make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+  };
+  auto wait = [&](int b, int use) {   // the MMAs of the use-th tile of buffer b (bounded)
     uint32_t done = 0;
     for (int it = 0; it < kWaitLimit && !done; ++it)
       asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                   : "=r"(done) : "r"(smem_u32(&mbar)), "r"(phase) : "memory");
-    phase ^= 1u;
-    ok = __syncthreads_and(done != 0);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                   : "=r"(done) : "r"(smem_u32(&mbar[b])), "r"(uint32_t(use) & 1u) : "memory");
+    return done != 0;
+  };
+  bool ok = true;
+  float sum = 0.0f;
+  for (int t0 = 0; t0 < ntiles; t0 += 2) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int t = t0 + b;
+      if (t < ntiles) {
+        unsigned char* sA = sop + b * kBuf;
+        unsigned char* sB = sA + kTM * kTK * 2;
+        if (t >= 2) ok = wait(b, (t >> 1) - 1) && ok;
+        int row, k;
+#pragma unroll
+        for (int i = 0; i < kNA; ++i) {
+          TileSource<AKC>::template place<kTM>(tid + kGemmThreads * i, row, k);
+          store(sA, row, k, ra[b][i]);
+        }
+#pragma unroll
+        for (int i = 0; i < kNB; ++i) {
+          TileSource<BKC>::template place<NT>(tid + kGemmThreads * i, row, k);
+          const float* v = rb[b][i];
+          store(sB, row, k, v);
+          if (BSUM) sum += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor cores
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (tid == 0) {
+#pragma unroll
+          for (int kk = 0; kk < kTK / 16; ++kk) {
+            const uint64_t ad = umma_desc(smem_u32(sA) + kk * 256, 128, (kTK / 8) * 128);
+            const uint64_t bd = umma_desc(smem_u32(sB) + kk * 256, 128, (kTK / 8) * 128);
+            const uint32_t acc = (t > 0 || kk > 0) ? 1u : 0u;
+            asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
+                         "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
+          }
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                           smem_u32(&mbar[b]))
+                       : "memory");
+        }
+        if (t + 2 < ntiles) fetch(b, (t + 2) * kTK);
+      }
+    }
   }
+  // the commit of the last tile covers every MMA before it
+  ok = wait((ntiles - 1) & 1, (ntiles - 1) >> 1) && ok;
+  ok = __syncthreads_and(ok);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (!ok && tid == 0 && status) atomicExch(status, 1);
-  // epilogue: warp w holds rows 32w .. 32w + 31 of the tile, 16 columns per load
-  const int gm = m0 + 32 * warp + lane;
-  for (int c0 = 0; c0 < kTN; c0 += 16) {
+  if (BSUM) {   // rows tid % 32 of the eight warps
+    float* part = reinterpret_cast<float*>(sop);   // the operand tiles are done with
+    part[tid] = sum;
+    __syncthreads();
+    if (tid < NT) {
+      sum = 0.0f;
+      for (int w = 0; w < kGemmThreads / 32; ++w) sum += part[w * NT + tid];
+      bsum[tid] = sum;
+    }
+    __syncthreads();
+  }
+  // epilogue: warps w and w + 4 hold rows 32 (w % 4) .. + 31 of the tile, half of the columns each, 16 per load
+  const int gm = m0 + 32 * (warp & 3) + lane;
+  for (int c0 = (NT / 2) * (warp >> 2), c1 = c0 + NT / 2; c0 < c1; c0 += 16) {
     uint32_t r[16];
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
                    "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(tmem + (uint32_t(32 * warp) << 16) + uint32_t(c0)));
+                 : "r"(tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(c0)));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    if (gm < M) {
+    const int nv = min(16, B.rows - (n0 + c0));
+    if (gm < A.rows && nv > 0) {
+      float v[16];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int gn = n0 + c0 + j;
-        if (gn < N) {
-          float v = ok ? __uint_as_float(r[j]) + (bias ? bias[gn] : 0.0f) : __int_as_float(0x7fc00000);
-          if (Z) Z[int64_t(gm) * ldc + gn] = v;
-          if (act) v = silu_f(v);
-          C[int64_t(gm) * ldc + gn] = v;
-        }
-      }
+      for (int j = 0; j < 16; ++j) v[j] = ok ? __uint_as_float(r[j]) : __int_as_float(0x7fc00000);
+      epi(gm, n0 + c0, v, nv);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(uint32_t(NT)) : "memory");
+}
+
+// nv <= 16 consecutive values, 16 bytes at a time where the row allows it
+__device__ __forceinline__ void store_row(float* dst, const float* v, int nv) {
+  if (nv == 16 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+#pragma unroll
+    for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(dst + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (j < nv) dst[j] = v[j];
+  }
+}
+
+// One layer forward: C = act(in W + bias), the pre-activations to Z if given.
+// With a target (the output layer of a training step) C instead receives the
+// gradient of the MSE, 2 (out - y) scale, and *loss the sum of scale (out - y)^2.
+__global__ void __launch_bounds__(kGemmThreads) layer_forward_kernel(int M, int N, int K, const float* __restrict__ in,
+                                                            const float* __restrict__ W, float* __restrict__ C,
+                                                            const float* __restrict__ bias, float* __restrict__ Z,
+                                                            int act, const float* __restrict__ target, float scale,
+                                                            float* __restrict__ loss, int* __restrict__ status) {
+  float s = 0.0f;
+  gemm_tile<kTN, false>(TileSource<true>(in, K, M, K), TileSource<false>(W, N, N, K), int(blockIdx.y) * kTM,
+                        int(blockIdx.x) * kTN, nullptr, status, [&](int gm, int gn, float* v, int nv) {
+              const int64_t at = int64_t(gm) * N + gn;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) v[j] += j < nv ? bias[gn + j] : 0.0f;
+              if (Z) store_row(Z + at, v, nv);
+              if (act) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = silu_f(v[j]);
+              }
+              if (target) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                  const float d = j < nv ? v[j] - target[at + j] : 0.0f;
+                  s += d * d;
+                  v[j] = 2.0f * d * scale;
+                }
+              }
+              store_row(C + at, v, nv);
+            });
+  if (target && loss) {
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(loss, s * scale);
+  }
+}
+
+// One layer backward: Z <- (dZ_next W^T) silu'(Z), in place (M rows, N = the
+// layer's width, K = the next layer's).
+__global__ void __launch_bounds__(kGemmThreads) layer_backward_kernel(int M, int N, int K, const float* __restrict__ dZn,
+                                                             const float* __restrict__ W, float* __restrict__ Z,
+                                                             int* __restrict__ status) {
+  gemm_tile<kTN, false>(TileSource<true>(dZn, K, M, K), TileSource<true>(W, K, N, K), int(blockIdx.y) * kTM,
+                        int(blockIdx.x) * kTN, nullptr, status, [&](int gm, int gn, float* v, int nv) {
+              float* z = Z + int64_t(gm) * N + gn;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) v[j] *= j < nv ? dsilu_f(z[j]) : 0.0f;
+              store_row(z, v, nv);
+            });
+}
+
+// Weight and bias gradients of every layer in one launch: block x is a tile of
+// one layer's dW = in^T dZ (M = fan-in, N = fan-out, K = batch). The contraction
+// is long and the output small (42 tiles of 128 x 32 for the 13-256-256-256-12
+// network), so a tile's k-tiles in sequence are what it takes; splitting the
+// batch over CTAs would be faster but sum in another order (8.6e-5 relative
+// from the sequential FP32 accumulation at 4,096 rows).
+struct GradLayer {
+  const float *in, *dz;
+  int fi, fo, tile0;   // first tile; tiles run over n, then m
+  int64_t off;         // of the layer's parameters [W b]
+};
+constexpr int kGradTN = 32;
+struct GradArgs {
+  int nl, B;
+  float* grad;
+  GradLayer layer[8];
+};
+__global__ void __launch_bounds__(kGemmThreads) weight_grad_kernel(const GradArgs a, int* __restrict__ status) {
+  __shared__ float bsum[kGradTN];
+  int l = 0;
+  while (l + 1 < a.nl && int(blockIdx.x) >= a.layer[l + 1].tile0) ++l;
+  const GradLayer& g = a.layer[l];
+  const int nt = (g.fo + kGradTN - 1) / kGradTN, t = int(blockIdx.x) - g.tile0;
+  const int m0 = t / nt * kTM, n0 = t % nt * kGradTN;
+  float* out = a.grad + g.off;
+  gemm_tile<kGradTN, true>(TileSource<false>(g.in, g.fi, g.fi, a.B), TileSource<false>(g.dz, g.fo, g.fo, a.B), m0, n0,
+                           bsum, status,
+                           [&](int gm, int gn, float* v, int nv) { store_row(out + int64_t(gm) * g.fo + gn, v, nv); });
+  if (m0 == 0 && int(threadIdx.x) < kGradTN && n0 + int(threadIdx.x) < g.fo)
+    out[int64_t(g.fi) * g.fo + n0 + threadIdx.x] = bsum[threadIdx.x];
 }
 
 // ---------------------------------------------------------------------------
@@ -256,11 +422,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
                  : "=r"(done) : "r"(bar), "r"(parity) : "memory");
   return done != 0;
-}
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);   // a in the low half (lower k)
-  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
@@ -563,34 +724,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_fused_forward_kernel(int
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(uint32_t(2 * kFusedMaxN)) : "memory");
 }
 
-// dZ = dH * silu'(Z), in place on dH.
-__global__ void silu_back_kernel(int64_t n, float* __restrict__ dH, const float* __restrict__ Z) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    dH[i] *= dsilu_f(Z[i]);
-}
-
-// MSE: dOut = 2 (out - y) / (B n_out); loss += sum (out - y)^2 / (B n_out).
-__global__ void mse_kernel(int64_t n, float scale, const float* __restrict__ out, const float* __restrict__ y,
-                           float* __restrict__ dout, float* __restrict__ loss) {
-  float s = 0.0f;
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    const float d = out[i] - y[i];
-    dout[i] = 2.0f * d * scale;
-    s += d * d;
-  }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0 && loss) atomicAdd(loss, s * scale);
-}
-
-// db[n] = sum_m dZ[m][n].
-__global__ void bias_grad_kernel(int M, int N, const float* __restrict__ dZ, float* __restrict__ db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.0f;
-  for (int m = 0; m < M; ++m) s += dZ[int64_t(m) * N + n];
-  db[n] = s;
-}
-
 // Adam (Kingma & Ba 2015, Algorithm 1), bias-corrected, FP32.
 __global__ void adam_kernel(int64_t n, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                             float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
@@ -689,26 +822,18 @@ std::vector<LayerOff> layers_of(const dlbchem_mlp* m) {
   return L;
 }
 
-cudaError_t gemm(bool ta, bool tb, int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C,
-                 int ldc, const float* bias, float* Z, int act, int* status, cudaStream_t s) {
-  if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;   // nothing to contract
-  dim3 grid((N + dlb::kTN - 1) / dlb::kTN, (M + dlb::kTM - 1) / dlb::kTM);
-  if (!ta && !tb) dlb::gemm_tc_kernel<false, false><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, Z, act, status);
-  else if (ta && !tb) dlb::gemm_tc_kernel<true, false><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, Z, act, status);
-  else if (!ta && tb) dlb::gemm_tc_kernel<false, true><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, Z, act, status);
-  else dlb::gemm_tc_kernel<true, true><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, Z, act, status);
-  return cudaGetLastError();
+dim3 tiles_of(int64_t rows, int cols) {
+  return dim3((cols + dlb::kTN - 1) / dlb::kTN, unsigned((rows + dlb::kTM - 1) / dlb::kTM));
 }
 
 // activation workspace: per hidden layer Z and H [cap x n_hidden], output
-// [cap x n_out], two gradient buffers [cap x max(n_hidden, n_out)].
+// (or its gradient) [cap x n_out].
 int ensure_act(dlbchem_mlp* m, int64_t batch) {
   if (batch <= m->cap) return DLBCHEM_OK;
   if (m->d_act) cudaFree(m->d_act);
   m->d_act = nullptr;
   m->cap = 0;
-  const int64_t wmax = std::max(m->n_hidden, m->n_out);
-  const int64_t per = 2 * int64_t(m->n_layers) * m->n_hidden + m->n_out + 2 * wmax;
+  const int64_t per = 2 * int64_t(m->n_layers) * m->n_hidden + m->n_out;
   if (cudaMalloc(&m->d_act, size_t(batch) * per * 4) != cudaSuccess) {
     m->d_act = nullptr;
     return mfail(m, DLBCHEM_OOM, "network activation allocation failed");
@@ -744,10 +869,6 @@ bool plan_fused(dlbchem_mlp* m) {
   for (int l = 0; l < f.nl; ++l) f.bias[l] = m->d_params + L[l].b;
   const int64_t last_bytes = int64_t(f.kp[f.nl - 1]) * f.np[f.nl - 1] * 2;
   f.res_bytes = last_bytes <= dlb::kFusedResident ? uint32_t(last_bytes) : 0u;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return false;
   return cudaFuncSetAttribute(dlb::mlp_fused_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               dlb::kFusedSmem) == cudaSuccess;
 }
@@ -773,10 +894,12 @@ cudaError_t forward_fused(dlbchem_mlp* m, int64_t B, const float* X, float* out,
   return cudaGetLastError();
 }
 
-// Forward; with keep the pre-activations are stored for the backward pass.
+// Forward; with keep the pre-activations are stored for the backward pass (and
+// with a target out receives the gradient of the MSE, *loss its value).
 // Without keep (inference) the fused whole-network kernel runs where the
 // shape allows it.
-cudaError_t forward(dlbchem_mlp* m, int64_t B, const float* X, float* out, bool keep, cudaStream_t s) {
+cudaError_t forward(dlbchem_mlp* m, int64_t B, const float* X, float* out, bool keep, cudaStream_t s,
+                    const float* target = nullptr, float scale = 0.0f, float* loss = nullptr) {
   if (!keep && m->fused_ok && m->fused_on) return forward_fused(m, B, X, out, s);
   const auto L = layers_of(m);
   const int64_t H = m->n_hidden;
@@ -788,8 +911,10 @@ cudaError_t forward(dlbchem_mlp* m, int64_t B, const float* X, float* out, bool 
     const bool last = li + 1 == int(L.size());
     float* dst = last ? out : Hs + int64_t(li) * B * H;
     float* z = (!last && keep) ? Zs + int64_t(li) * B * H : nullptr;
-    e = gemm(false, false, int(B), L[li].fo, L[li].fi, in, L[li].fi, m->d_params + L[li].w, L[li].fo, dst, L[li].fo,
-             m->d_params + L[li].b, z, last ? 0 : 1, m->d_status, s);
+    dlb::layer_forward_kernel<<<tiles_of(B, L[li].fo), dlb::kGemmThreads, 0, s>>>(int(B), L[li].fo, L[li].fi, in, m->d_params + L[li].w,
+                                                                   dst, m->d_params + L[li].b, z, last ? 0 : 1,
+                                                                   last ? target : nullptr, scale, loss, m->d_status);
+    e = cudaGetLastError();
     in = dst;
   }
   return e;
@@ -822,6 +947,10 @@ int dlbchem_mlp_create(int n_in, int n_hidden, int n_out, dlbchem_mlp** out) {
   for (int i = 0; i < n_in; ++i) norm[n_in + i] = 1.0f;
   for (int i = 0; i < n_out; ++i) norm[2 * n_in + n_out + i] = 1.0f;
   cudaMemcpy(m->d_norm, norm.data(), norm.size() * 4, cudaMemcpyHostToDevice);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    m->num_sms = 1;
   m->fused_ok = plan_fused(m);
   *out = m;
   return DLBCHEM_OK;
@@ -880,42 +1009,30 @@ int dlbchem_mlp_grad(dlbchem_mlp* m, int64_t B, const float* X, const float* Y, 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   float* g = grad ? grad : m->d_grad;
   const auto L = layers_of(m);
-  const int64_t H = m->n_hidden, wmax = std::max(m->n_hidden, m->n_out);
-  float* Zs = m->d_act;
+  const int64_t H = m->n_hidden;
+  float* Zs = m->d_act;                                  // pre-activations, then their gradients
   float* Hs = Zs + int64_t(m->n_layers) * B * H;
-  float* out = Hs + int64_t(m->n_layers) * B * H;
-  float* dA = out + B * m->n_out;
-  float* dB = dA + B * wmax;
-  cudaError_t e = forward(m, B, X, out, true, s);
-  if (e == cudaSuccess && loss) e = cudaMemsetAsync(loss, 0, 4, s);
-  if (e == cudaSuccess) {
-    const int64_t n = B * m->n_out;
-    dlb::mse_kernel<<<unsigned(std::min<int64_t>((n + 255) / 256, 1024)), 256, 0, s>>>(n, 1.0f / float(n), out, Y, dA,
-                                                                                     loss);
+  float* dout = Hs + int64_t(m->n_layers) * B * H;
+  cudaError_t e = loss ? cudaMemsetAsync(loss, 0, 4, s) : cudaSuccess;
+  if (e == cudaSuccess) e = forward(m, B, X, dout, true, s, Y, 1.0f / float(B * m->n_out), loss);
+  dlb::GradArgs a;
+  a.nl = int(L.size()); a.B = int(B); a.grad = g;
+  int tiles = 0;
+  for (int li = 0; li < a.nl; ++li) {
+    const int n = (L[li].fo + dlb::kGradTN - 1) / dlb::kGradTN * ((L[li].fi + dlb::kTM - 1) / dlb::kTM);
+    a.layer[li] = {li == 0 ? X : Hs + int64_t(li - 1) * B * H, li + 1 == a.nl ? dout : Zs + int64_t(li) * B * H,
+                   L[li].fi, L[li].fo, tiles, L[li].w};
+    tiles += n;
+  }
+  for (int li = a.nl - 1; li > 0 && e == cudaSuccess; --li) {
+    dlb::layer_backward_kernel<<<tiles_of(B, L[li].fi), dlb::kGemmThreads, 0, s>>>(int(B), L[li].fi, L[li].fo, a.layer[li].dz,
+                                                                     m->d_params + L[li].w,
+                                                                     Zs + int64_t(li - 1) * B * H, m->d_status);
     e = cudaGetLastError();
   }
-  float* dcur = dA;
-  float* dnext = dB;
-  for (int li = int(L.size()) - 1; li >= 0 && e == cudaSuccess; --li) {
-    const float* hin = li == 0 ? X : Hs + int64_t(li - 1) * B * H;
-    // dW = hin^T dZ  (M = fan_in, N = fan_out, K = B)
-    e = gemm(true, false, L[li].fi, L[li].fo, int(B), hin, L[li].fi, dcur, L[li].fo, g + L[li].w, L[li].fo, nullptr,
-             nullptr, 0, m->d_status, s);
-    if (e == cudaSuccess) {
-      dlb::bias_grad_kernel<<<(L[li].fo + 127) / 128, 128, 0, s>>>(int(B), L[li].fo, dcur, g + L[li].b);
-      e = cudaGetLastError();
-    }
-    if (li == 0 || e != cudaSuccess) break;
-    // dH_prev = dZ W^T  (M = B, N = fan_in, K = fan_out), then through SiLU
-    e = gemm(false, true, int(B), L[li].fi, L[li].fo, dcur, L[li].fo, m->d_params + L[li].w, L[li].fo, dnext,
-             L[li].fi, nullptr, nullptr, 0, m->d_status, s);
-    if (e == cudaSuccess) {
-      const int64_t n = B * H;
-      dlb::silu_back_kernel<<<unsigned(std::min<int64_t>((n + 255) / 256, 4096)), 256, 0, s>>>(
-          n, dnext, Zs + int64_t(li - 1) * B * H);
-      e = cudaGetLastError();
-    }
-    float* t = dcur; dcur = dnext; dnext = t;
+  if (e == cudaSuccess) {
+    dlb::weight_grad_kernel<<<unsigned(tiles), dlb::kGemmThreads, 0, s>>>(a, m->d_status);
+    e = cudaGetLastError();
   }
   return e == cudaSuccess ? DLBCHEM_OK : mfail(m, DLBCHEM_CUDA, cudaGetErrorString(e));
 }
