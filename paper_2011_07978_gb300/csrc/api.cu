@@ -151,7 +151,8 @@ bool parse_mech(const char* path, dlb::HostMech& m, std::string& err) {
 
 // Rounds of 32 entries, no target twice in a round. Each round takes the
 // (at most 32) targets with the most entries left, ties to the lower target,
-// which reaches the lower bound max(largest target count, ceil(n / 32)).
+// which reaches the lower bound max(largest target count, ceil(n / 32)); with
+// width 64, pairs of rounds in which no target occurs twice.
 // Per target the entries keep their input order, which fixes every
 // accumulation order.
 struct Entry {
@@ -161,7 +162,7 @@ struct Entry {
 };
 
 void build_rounds(const std::vector<Entry>& ents, uint32_t pad_word, std::vector<uint32_t>& words,
-                  std::vector<double>& coefs) {
+                  std::vector<double>& coefs, int width = 32) {
   std::map<int, std::vector<int>> by_t;
   for (int i = 0; i < int(ents.size()); ++i) by_t[ents[i].target].push_back(i);
   std::vector<std::pair<int, std::vector<int>*>> tl;   // (target, its entries)
@@ -177,14 +178,14 @@ void build_rounds(const std::vector<Entry>& ents, uint32_t pad_word, std::vector
     });
     int lane = 0;
     for (int i : idx) {
-      if (lane == 32 || next[i] == tl[i].second->size()) break;
+      if (lane == width || next[i] == tl[i].second->size()) break;
       const Entry& e = ents[(*tl[i].second)[next[i]++]];
       words.push_back(e.word);
       coefs.push_back(e.coef);
       ++lane;
       --left;
     }
-    for (; lane < 32; ++lane) { words.push_back(pad_word); coefs.push_back(0.0); }
+    for (; lane < width; ++lane) { words.push_back(pad_word); coefs.push_back(0.0); }
   }
 }
 
@@ -321,6 +322,8 @@ bool build_tables(const dlb::HostMech& hm, int wpc, std::vector<unsigned char>& 
                   std::vector<int>* order_out = nullptr) {
   const int nsp = hm.nsp, nrx = hm.nrx, N = nsp + 1, ld = N + 1;
   dm.nsp = nsp; dm.nrx = nrx; dm.N = N; dm.ld = ld; dm.wpc = wpc;
+  dm.three = 0;
+  for (const HostRxn& x : hm.rx) dm.three |= x.r.size() > 2 || x.p.size() > 2;
   if (N * ld + 2 >= 65536 || N > 256) { err = "mechanism too large (max 254 species)"; return false; }
   // species
   std::vector<double> W(nsp), iW(nsp), H0(nsp), cpa(nsp), hcpb(nsp), cpb(nsp), G0(nsp), G1(nsp), G2(nsp), G3(nsp), bW(nsp);
@@ -456,6 +459,26 @@ bool build_tables(const dlb::HostMech& hm, int wpc, std::vector<unsigned char>& 
     for (int k : x.p) nu[k] += 1;
     return nu;
   };
+  // Jacobian rounds in pairs unless a target is so frequent that most of the
+  // second rounds would be empty: a pair takes about 1.3 times a round
+  dm.tri_pair = 1;
+  {
+    long single = 0, pairs = 0;
+    for (int c = 0; c < nchunks; ++c) {
+      std::map<int, int> cnt;
+      int n = 0;
+      for (int r = c * CH; r < std::min(nrx, (c + 1) * CH); ++r) {
+        const auto& dl = distinct[r];
+        for (int k : shape[order[r]].ks)
+          for (int q : dl) { ++cnt[(1 + k) * ld + 1 + q]; ++n; }
+      }
+      int top = 0;
+      for (auto& kv : cnt) top = std::max(top, kv.second);
+      single += std::max(top, (n + 32 * wpc - 1) / (32 * wpc));
+      pairs += std::max(top, (n + 64 * wpc - 1) / (64 * wpc));
+    }
+    if (13 * pairs < 10 * single) dm.tri_pair = 2;
+  }
   for (int c = 0; c < nchunks; ++c) {
     std::map<int, int> mult, tmult;
     for (int r = c * CH; r < std::min(nrx, (c + 1) * CH); ++r)
@@ -490,7 +513,7 @@ bool build_tables(const dlb::HostMech& hm, int wpc, std::vector<unsigned char>& 
       incp.push_back(int32_t(inc.size() / 32));
       build_rounds(inc_w[w], pack_inc(nsp, 0, 0), inc, incc);
       trip.push_back(int32_t(tri.size() / 32));
-      build_rounds(tri_w[w], pack_tri(N * ld, 0), tri, tric);
+      build_rounds(tri_w[w], pack_tri(N * ld, 0), tri, tric, 32 * dm.tri_pair);
     }
   }
   incp.push_back(int32_t(inc.size() / 32));

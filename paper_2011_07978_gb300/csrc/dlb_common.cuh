@@ -58,6 +58,8 @@ __host__ __device__ inline uint32_t pack_tri(int e, int d) { return (uint32_t(e)
 
 struct DevMech {
   int nsp, nrx, N, ld, DS, wpc;
+  int tri_pair;           // Jacobian rounds per visit: 2 if pairs (2 i, 2 i + 1) have distinct targets, else 1
+  int three;              // some reaction has three molecules on a side
   // species
   const double *W, *iW, *H0, *cpa, *hcpb, *cpb, *G0, *G1, *G2, *G3, *bW;
   // reactions
@@ -119,7 +121,7 @@ struct IntegParams {
 struct WsLayout {
   int M, y0, f0, ys, fs, u, c, E, Einv, hk, wdot, vv, dwdT, uu, invd, q, dqdT, dlt, D, scal, perm;
   int M32, invd32, perm32, rr, dx, isc;   // mixed precision with more unknowns than threads only (else 0)
-  int w32, v, keys, rows;                 // refined solves with the FP32 inverse
+  int w32, v, xf, keys, rows;             // refined solves with the FP32 inverse
   int total;  // doubles per team (int and float arrays are counted in doubles)
 };
 
@@ -152,12 +154,13 @@ __host__ inline WsLayout make_layout(int nsp, int nrx, int CH, int N, int ld, in
   // refined solves: weights and right-hand side over the Jacobian-only arrays
   // dwdT .. dlt (dead from the assembly of one step to the next), keys and
   // published rows (dead during the rate evaluations too) behind them up to scal
-  L.w32 = L.v = L.keys = L.rows = 0;
+  L.w32 = L.v = L.xf = L.keys = L.rows = 0;
   if (N <= CH) {
     const int warps = CH / 32;
     auto vectors = [&](auto&& take2) {
       L.w32 = take2((N + 1) / 2);
       L.v = take2(CH / 2);
+      L.xf = take2((N + 1) / 2);
       L.keys = take2(warps);
       L.rows = take2(warps * CH);
     };

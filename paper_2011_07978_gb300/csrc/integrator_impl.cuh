@@ -131,6 +131,7 @@ struct InvScratch {
   float* rows;      // [2][WPC][NP] published rows
   unsigned* keys;   // [2][WPC]
   float* v;         // [NP] right-hand side in pivot order
+  float* xf;        // [N] first solution
 };
 
 struct WS {
@@ -159,7 +160,7 @@ __device__ __forceinline__ WS carve(double* base, const WsLayout& L) {
   w.perm32 = reinterpret_cast<int*>(base + L.perm32);
   w.rr = base + L.rr; w.dx = base + L.dx; w.isc = base + L.isc;
   w.inv = InvScratch{w.perm, reinterpret_cast<float*>(base + L.rows), reinterpret_cast<unsigned*>(base + L.keys),
-                     reinterpret_cast<float*>(base + L.v)};
+                     reinterpret_cast<float*>(base + L.v), reinterpret_cast<float*>(base + L.xf)};
   w.inv_isc = reinterpret_cast<float*>(base + L.w32);
   return w;
 }
@@ -345,6 +346,11 @@ __device__ __forceinline__ void reaction(const DevMech& m, const WS& w, const Mi
   const double a0 = w.c[mt.sp[0]];
   const double a1 = mt.nr > 1 ? w.c[mt.sp[1]] : 1.0;
   const double a2 = mt.nr > 2 ? w.c[mt.sp[2]] : 1.0;
+  // no reaction of the mechanism has three molecules on a side: the products
+  // by 1 are left out (uniform branches; 8 of 55 FP64 instructions with the
+  // Jacobian, 3 of 25 without)
+  const bool three = m.three != 0;
+  auto times = [three](double x, double y) { return three ? x * y : x; };
   double Mf = 1.0;
   if (mt.flags & RX_TB) {
     Mf = mx.Ctot;
@@ -360,42 +366,42 @@ __device__ __forceinline__ void reaction(const DevMech& m, const WS& w, const Mi
   }
   if (!JAC) {
     // q = Mq k_f (prod c_reac - prod E_reac prod (c/E)_prod); Einv holds c_k / E_k here
-    double d = a0 * (a1 * a2);
+    double d = a0 * times(a1, a2);
     if (mt.flags & RX_REV) {
       const double e1 = mt.nr > 1 ? w.E[mt.sp[1]] : 1.0;
       const double e2 = mt.nr > 2 ? w.E[mt.sp[2]] : 1.0;
       const double g1 = mt.np > 1 ? w.Einv[mt.sp[4]] : 1.0;
       const double g2 = mt.np > 2 ? w.Einv[mt.sp[5]] : 1.0;
-      d = fma(-(w.E[mt.sp[0]] * (e1 * e2)), w.Einv[mt.sp[3]] * (g1 * g2), d);
+      d = fma(-(w.E[mt.sp[0]] * times(e1, e2)), w.Einv[mt.sp[3]] * times(g1, g2), d);
     }
     qdst[rl] = (Mq * kf) * d;
     return;
   }
-  const double pf = kf * (a0 * (a1 * a2));
+  const double pf = kf * (a0 * times(a1, a2));
   double pr = 0.0, kr = 0.0, b0 = 1.0, b1 = 1.0, b2 = 1.0;
   if (mt.flags & RX_REV) {
     const double e1 = mt.nr > 1 ? w.E[mt.sp[1]] : 1.0;
     const double e2 = mt.nr > 2 ? w.E[mt.sp[2]] : 1.0;
     const double i1 = mt.np > 1 ? w.Einv[mt.sp[4]] : 1.0;
     const double i2 = mt.np > 2 ? w.Einv[mt.sp[5]] : 1.0;
-    kr = kf * ((w.E[mt.sp[0]] * (e1 * e2)) * (w.Einv[mt.sp[3]] * (i1 * i2)));
+    kr = kf * ((w.E[mt.sp[0]] * times(e1, e2)) * (w.Einv[mt.sp[3]] * times(i1, i2)));
     b0 = w.c[mt.sp[3]];
     b1 = mt.np > 1 ? w.c[mt.sp[4]] : 1.0;
     b2 = mt.np > 2 ? w.c[mt.sp[5]] : 1.0;
-    pr = kr * (b0 * (b1 * b2));
+    pr = kr * (b0 * times(b1, b2));
   }
   qdst[rl] = Mq * (pf - pr);
   double* D = w.D + rl * m.DS;
   for (int s2 = 0; s2 < mt.nds; ++s2) D[s2] = 0.0;
   // d/dc_j of the slot product = product of the other slots
   const double kfM = kf * Mq;
-  D[mt.ds[0]] += kfM * (a1 * a2);
-  if (mt.nr > 1) D[mt.ds[1]] += kfM * (a0 * a2);
+  D[mt.ds[0]] += kfM * times(a1, a2);
+  if (mt.nr > 1) D[mt.ds[1]] += kfM * times(a0, a2);
   if (mt.nr > 2) D[mt.ds[2]] += kfM * (a0 * a1);
   if (mt.flags & RX_REV) {
     const double krM = kr * Mq;
-    D[mt.ds[3]] -= krM * (b1 * b2);
-    if (mt.np > 1) D[mt.ds[4]] -= krM * (b0 * b2);
+    D[mt.ds[3]] -= krM * times(b1, b2);
+    if (mt.np > 1) D[mt.ds[4]] -= krM * times(b0, b2);
     if (mt.np > 2) D[mt.ds[5]] -= krM * (b0 * b1);
   }
   const int tb = (mt.flags & RX_TB) ? 1 : 0;
@@ -494,11 +500,19 @@ __device__ __forceinline__ void eval_rates(const DevMech& m, const Team<WPC>& tm
 #pragma unroll 1
     for (int r = tm.tid; r < nrx; r += TS) reaction<false, GEN>(m, w, mx, r, r, qa);
     tm.sync();
-    for (int rd = m.incp_all[tm.warp], r1 = m.incp_all[tm.warp + 1]; rd < r1; ++rd) {
-      const uint32_t e = m.inc_all[rd * 32 + tm.lane];
-      const int k = int(e >> 20), rr = int((e >> 4) & 0xffffu);
-      w.wdot[k] = fma(w.nutab[e & 15u], qa[rr], w.wdot[k]);
-      __syncwarp();
+    {
+      int rd = m.incp_all[tm.warp];
+      const int r1 = m.incp_all[tm.warp + 1];
+      const uint32_t* tab = m.inc_all + tm.lane;
+      uint32_t e = rd < r1 ? tab[rd * 32] : 0u, e2 = rd + 1 < r1 ? tab[rd * 32 + 32] : 0u;
+      for (; rd < r1; ++rd) {   // the words of two rounds ahead in flight
+        const uint32_t n2 = rd + 2 < r1 ? tab[rd * 32 + 64] : 0u;
+        const int k = int(e >> 20), rr = int((e >> 4) & 0xffffu);
+        w.wdot[k] = fma(w.nutab[e & 15u], qa[rr], w.wdot[k]);
+        __syncwarp();
+        e = e2;
+        e2 = n2;
+      }
     }
     tm.sync();
     if (m.nsplit) {
@@ -508,33 +522,80 @@ __device__ __forceinline__ void eval_rates(const DevMech& m, const Team<WPC>& tm
     return;
   }
   for (int k = tm.tid; k <= nsp; k += TS) {
-    w.wdot[k] = 0.0;
-    w.dwdT[k] = 0.0; w.uu[k] = 0.0;
+    w.wdot[k] = 0.0; w.dwdT[k] = 0.0; w.uu[k] = 0.0;
+    w.vv[k] = 0.0; w.ys[k] = 0.0; w.fs[k] = 0.0;   // ys, fs: free during the assembly
   }
   tm.sync();
   for (int c = 0; c < m.nchunks; ++c) {
     const int r = c * m.CH + tm.tid;
     if (r < nrx) reaction<true, GEN>(m, w, mx, r, tm.tid, w.q);
     tm.sync();
+    // Rounds go in pairs, with the table words of the next pair in flight: the
+    // two incidence rounds of a pair add to accumulators of their own (wdot,
+    // dwdT, uu and vv, ys, fs, added up after the chunks), the two Jacobian
+    // rounds have distinct targets (small mechanisms, whose rounds are as many
+    // as their most frequent target's entries, take one at a time). One round at a time was a chain of table
+    // load, gather, FMA and store, 780 and 470 cycles a round.
     const int ci = c * m.wpc + tm.warp;
-    for (int rd = m.incp[ci], r1 = m.incp[ci + 1]; rd < r1; ++rd) {
-      const uint32_t e = m.inc[rd * 32 + tm.lane];
-      const int k = int(e >> 20), rr = int((e >> 4) & 0xffffu);
-      const double nu = w.nutab[e & 15u];
-      w.wdot[k] = fma(nu, w.q[rr], w.wdot[k]);
-      w.dwdT[k] = fma(nu, w.dqdT[rr], w.dwdT[k]);
-      w.uu[k] = fma(nu, w.dlt[rr], w.uu[k]);
-      __syncwarp();
+    {
+      int rd = m.incp[ci];
+      const int r1 = m.incp[ci + 1];
+      const uint32_t* tab = m.inc + tm.lane;
+      uint32_t e0 = rd < r1 ? tab[rd * 32] : 0u, e1 = rd + 1 < r1 ? tab[rd * 32 + 32] : 0u;
+      while (rd < r1) {
+        const bool two = rd + 1 < r1;
+        const uint32_t n0 = rd + 2 < r1 ? tab[rd * 32 + 64] : 0u, n1 = rd + 3 < r1 ? tab[rd * 32 + 96] : 0u;
+        const int k0 = int(e0 >> 20), q0 = int((e0 >> 4) & 0xffffu);
+        const double nu0 = w.nutab[e0 & 15u];
+        if (two) {
+          const int k1 = int(e1 >> 20), q1 = int((e1 >> 4) & 0xffffu);
+          const double nu1 = w.nutab[e1 & 15u];
+          const double a0 = fma(nu0, w.q[q0], w.wdot[k0]), b0 = fma(nu0, w.dqdT[q0], w.dwdT[k0]);
+          const double c0 = fma(nu0, w.dlt[q0], w.uu[k0]);
+          const double a1 = fma(nu1, w.q[q1], w.vv[k1]), b1 = fma(nu1, w.dqdT[q1], w.ys[k1]);
+          const double c1 = fma(nu1, w.dlt[q1], w.fs[k1]);
+          w.wdot[k0] = a0; w.dwdT[k0] = b0; w.uu[k0] = c0;
+          w.vv[k1] = a1; w.ys[k1] = b1; w.fs[k1] = c1;
+        } else {
+          w.wdot[k0] = fma(nu0, w.q[q0], w.wdot[k0]);
+          w.dwdT[k0] = fma(nu0, w.dqdT[q0], w.dwdT[k0]);
+          w.uu[k0] = fma(nu0, w.dlt[q0], w.uu[k0]);
+        }
+        __syncwarp();
+        rd += 2;
+        e0 = n0;
+        e1 = n1;
+      }
     }
-    for (int rd = m.trip[ci], t1 = m.trip[ci + 1]; rd < t1; ++rd) {
-      const uint32_t e = m.tri[rd * 32 + tm.lane];
-      const double cf = m.tri_coef[rd * 32 + tm.lane];
-      const int tgt = int(e >> 16), d = int(e & 0xffffu);
-      w.M[tgt] = fma(cf, w.D[d], w.M[tgt]);
-      __syncwarp();
+    {
+      int rd = m.trip[ci];
+      const int t1 = m.trip[ci + 1], d = m.tri_pair;   // d: rounds per visit
+      const uint32_t* tab = m.tri + tm.lane;
+      const double* cof = m.tri_coef + tm.lane;
+      const int o = 32 * (d - 1);
+      uint32_t e0 = 0u, e1 = 0u;
+      double f0 = 0.0, f1 = 0.0;
+      if (rd < t1) { e0 = tab[rd * 32]; e1 = tab[rd * 32 + o]; f0 = cof[rd * 32]; f1 = cof[rd * 32 + o]; }
+      while (rd < t1) {
+        uint32_t n0 = 0u, n1 = 0u;
+        double g0 = 0.0, g1 = 0.0;
+        rd += d;
+        if (rd < t1) { n0 = tab[rd * 32]; n1 = tab[rd * 32 + o]; g0 = cof[rd * 32]; g1 = cof[rd * 32 + o]; }
+        const double a0 = fma(f0, w.D[e0 & 0xffffu], w.M[e0 >> 16]);
+        if (d == 2) w.M[e1 >> 16] = fma(f1, w.D[e1 & 0xffffu], w.M[e1 >> 16]);
+        w.M[e0 >> 16] = a0;
+        __syncwarp();
+        e0 = n0; e1 = n1; f0 = g0; f1 = g1;
+      }
     }
     tm.sync();
   }
+  for (int k = tm.tid; k < nsp; k += TS) {
+    w.wdot[k] += w.vv[k];
+    w.dwdT[k] += w.ys[k];
+    w.uu[k] += w.fs[k];
+  }
+  tm.sync();
 }
 
 // f = (f_T, f_Y): f_Y_k = W_k wdot_k / rho, f_T = -sum h_k wdot_k / (rho cp_mass).
@@ -612,8 +673,15 @@ __device__ __forceinline__ void assemble(const DevMech& m, const Team<WPC>& tm, 
   // T row: J_Tj = (1/cp) [ -sum_k (h_k/W_k) Shat_kj + (1/W_j)(-Hz - Q/(rho S) + Q cp_j/(rho cp)) ],
   // Hz = sum_k h_k z_k = Hu - Hv/(rho S)
   for (int j = tm.tid; j < nsp; j += TS) {
-    double hs = 0.0;
-    for (int k = 0; k < nsp; ++k) hs = fma(w.Einv[k], w.M[(1 + k) * ld + 1 + j], hs);
+    double hs = 0.0, hs1 = 0.0;
+    int k = 0;
+#pragma unroll 2
+    for (; k + 1 < nsp; k += 2) {
+      hs = fma(w.Einv[k], w.M[(1 + k) * ld + 1 + j], hs);
+      hs1 = fma(w.Einv[k + 1], w.M[(2 + k) * ld + 1 + j], hs1);
+    }
+    if (k < nsp) hs = fma(w.Einv[k], w.M[(1 + k) * ld + 1 + j], hs);
+    hs += hs1;
     const double cpj = cp_of<GEN>(m, j, mx.T);
     const double bracket = fma(Q * cpj, mx.irho * icpm, -fma(Q, irS, Hz));
     const double JT = icpm * fma(m.iW[j], bracket, -hs);
@@ -625,11 +693,24 @@ __device__ __forceinline__ void assemble(const DevMech& m, const Team<WPC>& tm, 
     w.M[0] = iso ? ihg : ihg - JTT;
   }
   tm.sync();
-  // species block: M = delta/(h gamma) - (Shat_kj + r_k / W_j); warps take rows, lanes columns
-  for (int k = tm.warp; k < nsp; k += WPC) {
-    const double rk = w.E[k];
-    double* row = w.M + (1 + k) * ld + 1;
-    for (int j = tm.lane; j < nsp; j += 32) row[j] = fma(-rk, m.iW[j], -row[j]);
+  // species block: M = delta/(h gamma) - (Shat_kj + r_k / W_j); lanes take
+  // columns, warps rows, the rows four at a time (independent updates)
+  for (int j = tm.lane; j < nsp; j += 32) {
+    const double iw = m.iW[j];
+    double* col = w.M + 1 + j;
+    int k = tm.warp;
+    for (; k + 3 * WPC < nsp; k += 4 * WPC) {
+      double* p0 = col + (1 + k) * ld;
+      double* p1 = p0 + WPC * ld;
+      double* p2 = p1 + WPC * ld;
+      double* p3 = p2 + WPC * ld;
+      const double v0 = *p0, v1 = *p1, v2 = *p2, v3 = *p3;
+      *p0 = fma(-w.E[k], iw, -v0);
+      *p1 = fma(-w.E[k + WPC], iw, -v1);
+      *p2 = fma(-w.E[k + 2 * WPC], iw, -v2);
+      *p3 = fma(-w.E[k + 3 * WPC], iw, -v3);
+    }
+    for (; k < nsp; k += WPC) col[(1 + k) * ld] = fma(-w.E[k], iw, -col[(1 + k) * ld]);
   }
   tm.sync();
   for (int k = tm.tid; k < nsp; k += TS) w.M[(1 + k) * (ld + 1)] += ihg;
@@ -1129,12 +1210,34 @@ __device__ __noinline__ bool invert(const Team<WPC> tm, const double* M, int N, 
   return true;
 }
 
+// r - a x with a rounded to two floats (53 to 48 bits, integer operations) and
+// x a float: r is the unevaluated sum s + low of two floats, the sum of the
+// rounding errors of s goes to low (Knuth's two-sum, Dekker's product).
+__device__ __forceinline__ void sub_product(float& s, float& low, double a, float x) {
+  const unsigned hi = unsigned(__double2hiint(a)), lo = unsigned(__double2loint(a));
+  const float h = low_float(a);
+  // the 29 bits below h times 2^(exponent - 1075), the sign of a; dropped below 2^-74
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  const float unit = __uint_as_float(e > 948u && e < 1151u ? (hi & 0x80000000u) | ((e - 948u) << 23) : 0u);
+  const float l = __fmul_rn(float(lo & 0x1fffffffu), unit);
+  const float p = __fmul_rn(h, x);
+  const float q = fmaf(l, x, fmaf(h, x, -p));
+  const float d = __fsub_rn(s, p), b = __fsub_rn(d, s);
+  const float t = __fsub_rn(__fsub_rn(s, __fsub_rn(d, b)), __fadd_rn(p, b));
+  s = d;
+  low = __fadd_rn(low, __fsub_rn(t, q));
+}
+
 // x = M^-1 b by the refinement above. With the error weights isc = 1/sc, dmax
 // = max |d_i| isc_i of the last correction d and xmax = max |x_i| isc_i:
 //  - tight (the default, FP64 accuracy): done when dmax <= 2^-30 xmax. The
 //    correction's own relative error is that of a product with X, 2^-24 cond,
 //    so what is left is below 2^-54 cond, the error of an FP64 LU. Two
-//    rounds reach it unless 2^-24 cond > 2^-15; at most eight are tried.
+//    rounds reach it unless 2^-24 cond > 2^-15; at most eight are tried. The
+//    first round's x is a float and its residual cancels to 2^-24 of b, so 2^-45
+//    of |M||x| is enough for it: it is taken in paired floats, beside the FP64
+//    unit instead of on it (108 fewer FP64 instructions per solve at 54
+//    unknowns; the FP32 pipe runs at full rate next to a busy FP64 unit).
 //  - mixed precision (the caller's choice): done when the error left, dmax
 //    rho / (1 - rho), is below 1e-6, with rho estimated by dmax / xmax after
 //    the first correction and by the ratio of successive corrections after
@@ -1143,6 +1246,7 @@ __device__ __noinline__ bool invert(const Team<WPC> tm, const double* M, int N, 
 template <int WPC, int NP>
 __device__ __noinline__ bool solve_inverse(const Team<WPC> tm, const double* M, int N, int ld, const InvScratch sc,
                                            const float4* X4, const double* b, double* x, const float* isc, bool tight) {
+  constexpr bool kPairs = NP > 32;   // below, the FP64 residual is short (0.4 kcycles less per solve at 11 unknowns)
   const int t = tm.tid;
   const bool has = t < N;
   const int i = min(t, N - 1);
@@ -1169,20 +1273,41 @@ __device__ __noinline__ bool solve_inverse(const Team<WPC> tm, const double* M, 
   if (has) sc.v[at] = low_float(bi);
   else if (t < NP) sc.v[t] = 0.f;
   tm.sync();
-  double xi = double(apply());
-  if (has) x[i] = xi;
+  const float x0 = apply();
+  double xi = double(x0);
+  if (has) {
+    x[i] = xi;
+    if (kPairs) sc.xf[i] = x0;
+  }
   tm.sync();
   float prev = 0.f;
   for (int it = 0; it < (tight ? 8 : 3); ++it) {
-    double r0 = bi, r1 = 0.0;
-    int j = 0;
+    float rf;
+    if (kPairs && tight && it == 0) {
+      float s = low_float(bi), low = 0.f;
+      float s1 = low_float(bi - double(s)), low1 = 0.f;   // b's low part opens the second sum
+      int j = 0;
+#pragma unroll 2
+      for (; j + 1 < N; j += 2) {
+        sub_product(s, low, row[j], sc.xf[j]);
+        sub_product(s1, low1, row[j + 1], sc.xf[j + 1]);
+      }
+      if (j < N) sub_product(s, low, row[j], sc.xf[j]);
+      // s + s1 cancel: keep the rounding error of their sum
+      const float d = __fadd_rn(s, s1), b = __fsub_rn(d, s);
+      rf = d + ((__fsub_rn(s, __fsub_rn(d, b)) + __fsub_rn(s1, b)) + (low + low1));
+    } else {
+      double r0 = bi, r1 = 0.0;
+      int j = 0;
 #pragma unroll 4
-    for (; j + 1 < N; j += 2) {
-      r0 = fma(-row[j], x[j], r0);
-      r1 = fma(-row[j + 1], x[j + 1], r1);
+      for (; j + 1 < N; j += 2) {
+        r0 = fma(-row[j], x[j], r0);
+        r1 = fma(-row[j + 1], x[j + 1], r1);
+      }
+      if (j < N) r0 = fma(-row[j], x[j], r0);
+      rf = low_float(r0 + r1);
     }
-    if (j < N) r0 = fma(-row[j], x[j], r0);
-    if (has) sc.v[at] = low_float(r0 + r1);
+    if (has) sc.v[at] = rf;
     tm.sync();
     const float d = apply();
     xi += double(d);
@@ -1397,11 +1522,20 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
         acc = fma(r, r, acc);
         w.ys[i] = yn;
       }
-      double errn = sqrt(tm.sum(acc) * iN);
-      if (!ok) errn = nan("");
+      const double err2 = tm.sum(acc) * iN;
+      // one warp takes the square roots (60 FP64 instructions) for the team;
+      // 0.9 errn^(-1/4) as rsqrt(sqrt(errn)): within 2 ulp of pow
+      if (tm.warp == 0) {
+        double errn = sqrt(err2);
+        if (!ok) errn = nan("");
+        const double fac = isfinite(errn) ? 0.9 * rsqrt(sqrt(errn)) : 0.2;
+        if (tm.lane == 0) { w.scal[26] = errn; w.scal[27] = fac; }
+      }
+      tm.sync();
+      const double errn = w.scal[26];
+      double fac = fmax(0.2, w.scal[27]);
       if (errn <= 1.0) {
-        // errn^(-1/4) as rsqrt(sqrt(errn)): within 2 ulp of pow, at a fraction of its FP64 work
-        double fac = fmin(5.0, fmax(0.2, 0.9 * rsqrt(sqrt(errn))));
+        fac = fmin(5.0, fac);
         if (rejected_last) fac = fmin(fac, 1.0);
         t = (t + h >= dt) ? dt : t + h;
         for (int i = tm.tid; i < N; i += TS) w.y0[i] = w.ys[i];
@@ -1409,7 +1543,6 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
         rejected_last = false;
         h *= fac;
       } else {
-        const double fac = isfinite(errn) ? fmax(0.2, 0.9 * rsqrt(sqrt(errn))) : 0.2;
         rejected_last = true;
         h *= fac;
       }
