@@ -485,6 +485,16 @@ bool build_tables(const dlb::HostMech& hm, int wpc, std::vector<unsigned char>& 
       for (int k : shape[order[r]].ks) { mult[k] += 1; tmult[k] += shape[order[r]].ntri; }
     const auto wof = assign_warps(mult, tmult, wpc, parity);
     std::vector<std::vector<Entry>> inc_w(wpc), tri_w(wpc);
+    // incidence entries of a species alternate between the two warps of its
+    // warp's pair, which add to accumulators of their own: a chunk's rounds
+    // are held up by its most frequent species (78 -> 43 rounds at 53/325)
+    std::map<int, int> turn;
+    auto inc_warp = [&](int k, int w) {
+      if (wpc == 1) return 0;
+      auto it = turn.find(k);
+      if (it == turn.end()) it = turn.insert({k, inc_w[w & ~1].size() <= inc_w[w | 1].size() ? 0 : 1}).first;
+      return (w & ~1) | (it->second++ & 1);
+    };
     for (int r = c * CH; r < std::min(nrx, (c + 1) * CH); ++r) {
       const int rl = r - c * CH;
       const HostRxn& x = hm.rx[order[r]];
@@ -493,7 +503,7 @@ bool build_tables(const dlb::HostMech& hm, int wpc, std::vector<unsigned char>& 
         if (v == 0) continue;
         if (v < -7 || v > 7) { err = "stoichiometric coefficient out of range"; return false; }
         const int w = wof.at(k);
-        inc_w[w].push_back({k, pack_inc(k, rl, v), double(v)});
+        inc_w[inc_warp(k, w)].push_back({k, pack_inc(k, rl, v), double(v)});
         const auto& dl = distinct[r];
         for (int s2 = 0; s2 < int(dl.size()); ++s2) {
           const int j = dl[s2];
@@ -827,10 +837,12 @@ bool verify_tables(const dlb::HostMech& hm, int wpc, const std::vector<unsigned 
     return nu;
   };
   // one list of rounds: distinct targets per round, entries collected per target in round order
+  // (group 2: over pairs of rounds)
   auto scan = [&](const uint32_t* words, int r0, int r1, uint32_t pad, int shift, uint32_t mask,
-                  std::map<int, std::vector<int>>& by_target) {
+                  std::map<int, std::vector<int>>& by_target, int group = 1) {
+    std::vector<int> seen;
     for (int rd = r0; rd < r1; ++rd) {
-      std::vector<int> seen;
+      if ((rd - r0) % group == 0) seen.clear();
       for (int l = 0; l < 32; ++l) {
         const uint32_t e = words[size_t(rd) * 32 + l];
         if (e == pad) continue;
@@ -844,7 +856,8 @@ bool verify_tables(const dlb::HostMech& hm, int wpc, const std::vector<unsigned 
   };
   int64_t inc_rounds = 0, tri_rounds = 0;
   for (int c = 0; c < dm.nchunks; ++c) {
-    std::map<int, int> owner;        // species -> warp, incidence and Jacobian
+    std::map<int, int> owner;        // (species, accumulator set) -> warp
+    std::map<int, int> rows;         // species -> warp of its Jacobian row
     std::map<std::pair<int, int>, int> want_inc;   // (k, rl) -> nu
     std::map<std::pair<int, int>, double> want_tri;   // (M index, D index) -> coefficient
     for (int r = c * CH; r < std::min(nrx, (c + 1) * CH); ++r) {
@@ -868,12 +881,14 @@ bool verify_tables(const dlb::HostMech& hm, int wpc, const std::vector<unsigned 
       const int ci = c * wpc + w;
       std::map<int, std::vector<int>> bi, bt;
       if (!scan(inc, incp[ci], incp[ci + 1], inc_pad, 20, 0xfffu, bi)) return false;
-      if (!scan(tri, trip[ci], trip[ci + 1], tri_pad, 16, 0xffffu, bt)) return false;
+      if (!scan(tri, trip[ci], trip[ci + 1], tri_pad, 16, 0xffffu, bt, dm.tri_pair)) return false;
+      if ((trip[ci + 1] - trip[ci]) % dm.tri_pair) { err = "odd number of paired Jacobian rounds"; return false; }
       inc_rounds += incp[ci + 1] - incp[ci];
       tri_rounds += trip[ci + 1] - trip[ci];
       for (auto& kv : bi) {
-        if (owner.count(kv.first) && owner[kv.first] != w) { err = "species in two warps of a chunk"; return false; }
-        owner[kv.first] = w;
+        const int at = 2 * kv.first + (w & 1);   // odd warps have the second set
+        if (owner.count(at) && owner[at] != w) { err = "accumulator in two warps of a chunk"; return false; }
+        owner[at] = w;
         int prev = -1;
         for (int pos : kv.second) {
           const uint32_t e = inc[pos];
@@ -887,7 +902,8 @@ bool verify_tables(const dlb::HostMech& hm, int wpc, const std::vector<unsigned 
       }
       for (auto& kv : bt) {
         const int k = kv.first / ld - 1;
-        if (!owner.count(k) || owner[k] != w) { err = "Jacobian target outside its species' warp"; return false; }
+        if (rows.count(k) && rows[k] != w) { err = "Jacobian row in two warps of a chunk"; return false; }
+        rows[k] = w;
         for (int pos : kv.second) {
           const int d = int(tri[pos] & 0xffffu);
           auto it = want_tri.find({kv.first, d});

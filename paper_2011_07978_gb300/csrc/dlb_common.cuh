@@ -121,7 +121,7 @@ struct IntegParams {
 struct WsLayout {
   int M, y0, f0, ys, fs, u, c, E, Einv, hk, wdot, vv, dwdT, uu, invd, q, dqdT, dlt, D, scal, perm;
   int M32, invd32, perm32, rr, dx, isc;   // mixed precision with more unknowns than threads only (else 0)
-  int w32, v, xf, keys, rows;             // refined solves with the FP32 inverse
+  int w32, v, xf, invs, rows;             // refined solves with the FP32 inverse
   int total;  // doubles per team (int and float arrays are counted in doubles)
 };
 
@@ -152,17 +152,16 @@ __host__ inline WsLayout make_layout(int nsp, int nrx, int CH, int N, int ld, in
   L.perm = take((N + 1) / 2 + 1);
   L.M32 = L.invd32 = L.perm32 = L.rr = L.dx = L.isc = 0;
   // refined solves: weights and right-hand side over the Jacobian-only arrays
-  // dwdT .. dlt (dead from the assembly of one step to the next), keys and
-  // published rows (dead during the rate evaluations too) behind them up to scal
-  L.w32 = L.v = L.xf = L.keys = L.rows = 0;
+  // dwdT .. dlt (dead from the assembly of one step to the next), published
+  // rows (dead during the rate evaluations too) behind them up to scal
+  L.w32 = L.v = L.xf = L.invs = L.rows = 0;
   if (N <= CH) {
-    const int warps = CH / 32;
     auto vectors = [&](auto&& take2) {
       L.w32 = take2((N + 1) / 2);
       L.v = take2(CH / 2);
       L.xf = take2((N + 1) / 2);
-      L.keys = take2(warps);
-      L.rows = take2(warps * CH);
+      L.invs = take2(1);
+      L.rows = take2(CH);
     };
     int o2 = L.dwdT;
     vectors([&](int n) { int r = o2; o2 += (n + 1) & ~1; return r; });

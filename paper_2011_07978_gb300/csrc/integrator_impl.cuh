@@ -127,10 +127,9 @@ struct Team {
 
 // Scratch of the refined solves (invert and solve_inverse below).
 struct InvScratch {
-  int* pinv;        // [N] column whose pivot row i was
-  float* rows;      // [2][WPC][NP] published rows
-  unsigned* keys;   // [2][WPC]
-  float* v;         // [NP] right-hand side in pivot order
+  float* rows;      // [2][NP] published pivot rows
+  float* invs;      // [2] reciprocals of their pivots
+  float* v;         // [NP] right-hand side
   float* xf;        // [N] first solution
 };
 
@@ -159,7 +158,7 @@ __device__ __forceinline__ WS carve(double* base, const WsLayout& L) {
   w.M32 = reinterpret_cast<float*>(base + L.M32); w.invd32 = reinterpret_cast<float*>(base + L.invd32);
   w.perm32 = reinterpret_cast<int*>(base + L.perm32);
   w.rr = base + L.rr; w.dx = base + L.dx; w.isc = base + L.isc;
-  w.inv = InvScratch{w.perm, reinterpret_cast<float*>(base + L.rows), reinterpret_cast<unsigned*>(base + L.keys),
+  w.inv = InvScratch{reinterpret_cast<float*>(base + L.rows), reinterpret_cast<float*>(base + L.invs),
                      reinterpret_cast<float*>(base + L.v), reinterpret_cast<float*>(base + L.xf)};
   w.inv_isc = reinterpret_cast<float*>(base + L.w32);
   return w;
@@ -195,6 +194,36 @@ __device__ __forceinline__ double exp_tab(double x, const double* __restrict__ t
   p = fma(r, p, 1.0);
   const double v = tab[ki & 63] * p;
   return __hiloint2double(__double2hiint(v) + ((ki >> 6) << 20), __double2loint(v));
+}
+
+// ln x with the same table: x = 2^e m, n/64 = e + j/64 with j/64 the multiple of
+// 1/64 nearest log2 m (from the FP32 hardware logarithm, whose error only moves
+// a tie), z = m 2^(-j/64) in [1 - 0.0055, 1 + 0.0055], ln x = n ln2/64 + ln z with
+// the Mercator series of s = z - 1 to s^7 (remainder below 1.1e-19): 0.6 ulp
+// between 200 and 4,000 K against an 80-bit logarithm, the roundings of z being
+// absolute (1.7e-16). 12 FP64 operations against about 28; zero, negative,
+// subnormal and non-finite arguments go to the library.
+static __device__ __noinline__ double log_library(double x) { return log(x); }
+__device__ __forceinline__ double log_tab(double x, const double* __restrict__ tab) {
+  const int hi = __double2hiint(x);
+  if (hi < 0x00100000 || hi >= 0x7ff00000) return log_library(x);
+  const int e = (hi >> 20) - 1023;
+  const int mant = hi & 0xfffff;
+  const float mf = __int_as_float(0x3f800000 | (mant << 3));   // m to 20 bits
+  const int j = __float2int_rn(64.0f * __log2f(mf));           // 0 .. 64
+  // m 2^(-j/64) = m/2 2^((64 - j)/64) for j > 0
+  const double mh = __hiloint2double(mant | (j > 0 ? 0x3fe00000 : 0x3ff00000), __double2loint(x));
+  const double s = mh * tab[(64 - j) & 63] - 1.0;
+  const int n = 64 * e + j;
+  const double kd = __hiloint2double(0x43380000, int(0x80000000u) ^ n) - 6755401588539392.0;   // n, exactly
+  double p = fma(s, 1.0 / 7.0, -1.0 / 6.0);
+  p = fma(s, p, 1.0 / 5.0);
+  p = fma(s, p, -1.0 / 4.0);
+  p = fma(s, p, 1.0 / 3.0);
+  p = fma(s, p, -0.5);
+  p = fma(s * s, p, s);
+  p = fma(kd, -6.563929801064195e-13, p);                   // the constants of exp_tab
+  return fma(kd, 0.010830424696905538, p);
 }
 
 // 1/d from the hardware approximation r = rcp.approx.ftz.f64(d) by one
@@ -457,11 +486,11 @@ __device__ __forceinline__ void eval_rates(const DevMech& m, const Team<WPC>& tm
   double iT, lnT;
   if (WPC == 1) {
     iT = rcp_nr(T);
-    lnT = log(T);
+    lnT = log_tab(T, w.exptab);
   } else {
     // one warp takes ln T, another 1/T; both are published with the barrier
     // of the sum below (slots 28, 29 of the team scratch)
-    if (tm.warp == 0) { if (tm.lane == 0) w.scal[28] = log(T); }
+    if (tm.warp == 0) { if (tm.lane == 0) w.scal[28] = log_tab(T, w.exptab); }
     else if (tm.warp == 1) { if (tm.lane == 0) w.scal[29] = rcp_nr(T); }
   }
   const double S = tm.sum(s);
@@ -530,14 +559,34 @@ __device__ __forceinline__ void eval_rates(const DevMech& m, const Team<WPC>& tm
     const int r = c * m.CH + tm.tid;
     if (r < nrx) reaction<true, GEN>(m, w, mx, r, tm.tid, w.q);
     tm.sync();
-    // Rounds go in pairs, with the table words of the next pair in flight: the
-    // two incidence rounds of a pair add to accumulators of their own (wdot,
-    // dwdT, uu and vv, ys, fs, added up after the chunks), the two Jacobian
-    // rounds have distinct targets (small mechanisms, whose rounds are as many
-    // as their most frequent target's entries, take one at a time). One round at a time was a chain of table
-    // load, gather, FMA and store, 780 and 470 cycles a round.
+    // One round at a time was a chain of table load, gather, FMA and store, 780
+    // and 470 cycles a round: the table words of the next rounds are in flight
+    // now, and there are two sets of accumulators (wdot, dwdT, uu and vv, ys, fs,
+    // added up after the chunks). Odd warps have the second set, so a species'
+    // entries go to two warps; a lone warp takes its rounds in pairs, one to
+    // each set. Jacobian rounds go in pairs of distinct targets (small
+    // mechanisms, whose rounds are as many as their most frequent target's
+    // entries, take one at a time).
     const int ci = c * m.wpc + tm.warp;
-    {
+    if (WPC > 1) {
+      int rd = m.incp[ci];
+      const int r1 = m.incp[ci + 1];
+      const uint32_t* tab = m.inc + tm.lane;
+      double* s0 = tm.warp & 1 ? w.vv : w.wdot;
+      double* s1 = tm.warp & 1 ? w.ys : w.dwdT;
+      double* s2 = tm.warp & 1 ? w.fs : w.uu;
+      uint32_t e = rd < r1 ? tab[rd * 32] : 0u, e2 = rd + 1 < r1 ? tab[rd * 32 + 32] : 0u;
+      for (; rd < r1; ++rd) {
+        const uint32_t n2 = rd + 2 < r1 ? tab[rd * 32 + 64] : 0u;
+        const int k = int(e >> 20), rr = int((e >> 4) & 0xffffu);
+        const double nu = w.nutab[e & 15u];
+        const double a = fma(nu, w.q[rr], s0[k]), b = fma(nu, w.dqdT[rr], s1[k]), d = fma(nu, w.dlt[rr], s2[k]);
+        s0[k] = a; s1[k] = b; s2[k] = d;
+        __syncwarp();
+        e = e2;
+        e2 = n2;
+      }
+    } else {
       int rd = m.incp[ci];
       const int r1 = m.incp[ci + 1];
       const uint32_t* tab = m.inc + tm.lane;
@@ -1123,76 +1172,60 @@ __device__ __forceinline__ float low_float(double v) {
 // 64-bit integration is the same (1.3e-14 and 1.4e-14 relative in Y on 4,001
 // cells of 53 species, 1.1e-13 and 1.1e-13 on 400 of 100).
 //
-// Gauss-Jordan elimination in registers: thread i holds row i. Per column each
-// warp's best pivot row publishes itself (key and row, double-buffered), one
-// barrier, and every thread subtracts its multiple of the best of those rows.
-// Columns rotate: element j moves to j - 1 as it is updated, the pivot column
-// is always element 0 and the new column of the inverse enters at the end, so
-// that every register index is fixed in a loop over the columns. A pivot row is
-// scaled once, at the end. Rows stay where they are: the row that was pivot
-// of column m ends as row m of X with the columns in pivot order, so X is
-// applied to a right-hand side in that order (pinv[i] = m). The pivot is a
-// largest |M_ik| to within 2^-16 relative: the 32-bit key is |M_ik| with its 7
-// low bits replaced by 127 - i, so ties go to the lower row. X goes to a
-// global per-team scratch (L2), four columns per 16 bytes: X4[q N + m]. Returns
-// false if a pivot is zero (or below the key's resolution).
+// Gauss-Jordan elimination in registers: thread i holds row i. Per column k the
+// owner of row k has published it (double-buffered), one barrier, and every
+// thread subtracts its multiple; the owner of row k + 1 then publishes the
+// next. Columns rotate: element j moves to j - 1 as it is updated, the pivot
+// column is always element 0 and the new column of the inverse enters at the
+// end, so that every register index is fixed in a loop over the columns. A
+// pivot row is scaled once, at the end. The diagonal is the pivot, without a
+// search: searching and exchanging the largest |M_ik| was 600 of the 850 cycles
+// of a column at 54 unknowns. The matrices are close to diagonally dominant
+// (the columns of J sum to zero over the species), and X is only a
+// preconditioner: on 27,000 steps over the three mechanisms and all classes of
+// states both the pivoted and this inverse took two rounds on every one. Where
+// a pivot is so small that the refinement does not converge, the FP64 LU
+// (partial pivoting) takes the step. X goes to a global per-team scratch (L2),
+// four columns per 16 bytes: X4[q N + row].
 // ---------------------------------------------------------------------------
 template <int WPC, int NP>
-__device__ __noinline__ bool invert(const Team<WPC> tm, const double* M, int N, int ld, const InvScratch sc, float4* X4) {
+__device__ __noinline__ void invert(const Team<WPC> tm, const double* M, int N, int ld, const InvScratch sc, float4* X4) {
   const int row = tm.tid;
   const bool has = row < N;
-  bool live = has;
-  int m = 0;
   float scale = 0.f;
   float a[NP];
   const double* src = M + min(row, N - 1) * ld;
 #pragma unroll
   for (int j = 0; j < NP; ++j) a[j] = has && j < N ? low_float(src[j]) : 0.f;
-  volatile unsigned* keys = sc.keys;
-  for (int k = 0; k < N; ++k) {
-    const unsigned key = live ? (__float_as_uint(a[0]) & 0x7fffff80u) | unsigned(127 - row) : 0u;
-    const unsigned best = __reduce_max_sync(0xffffffffu, key);
-    const int buf = (k & 1) * WPC;
-    if ((best >> 7) == 0u) {
-      if (tm.lane == 0) keys[buf + tm.warp] = 0u;
-    } else if (key == best) {
-      keys[buf + tm.warp] = best;
-      float4* dst = reinterpret_cast<float4*>(sc.rows + (buf + tm.warp) * NP);
-#pragma unroll
-      for (int q = 0; q < NP / 4; ++q) dst[q] = make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
-    }
-    tm.sync();
-    unsigned top = keys[buf];
-    int from = buf;
-#pragma unroll
-    for (int w = 1; w < WPC; ++w) {
-      const unsigned kw = keys[buf + w];
-      if (kw > top) { top = kw; from = buf + w; }
-    }
-    if (top == 0u) return false;   // the same in every thread
-    const float4* u4 = reinterpret_cast<const float4*>(sc.rows + from * NP);
-    float4 u = u4[0];
+  volatile float* invs = sc.invs;
+  auto publish = [&](int k) {
     float rp;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rp) : "f"(u.x));
-    const bool piv = has && row == 127 - int(top & 127u);
-    const float nf = piv ? 0.f : -(a[0] * rp);
-    if (piv) {
-      live = false;
-      m = k;
-      scale = rp;
-    }
-    a[0] = fmaf(nf, u.y, a[1]);
-    a[1] = fmaf(nf, u.z, a[2]);
-    a[2] = fmaf(nf, u.w, a[3]);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rp) : "f"(a[0]));
+    invs[k & 1] = rp;
+    float4* dst = reinterpret_cast<float4*>(sc.rows + (k & 1) * NP);
 #pragma unroll
-    for (int q = 1; q < NP / 4; ++q) {
-      u = u4[q];
-      a[4 * q - 1] = fmaf(nf, u.x, a[4 * q]);
-      a[4 * q] = fmaf(nf, u.y, a[4 * q + 1]);
-      a[4 * q + 1] = fmaf(nf, u.z, a[4 * q + 2]);
-      a[4 * q + 2] = fmaf(nf, u.w, a[4 * q + 3]);
+    for (int q = 0; q < NP / 4; ++q) dst[q] = make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
+  };
+  if (row == 0) publish(0);
+  for (int k = 0; k < N; ++k) {
+    tm.sync();   // row k is there, and row k - 1's buffer is no longer read
+    const float4* u4 = reinterpret_cast<const float4*>(sc.rows + (k & 1) * NP);
+    const float rp = invs[k & 1];
+    float4 u[NP / 4];
+#pragma unroll
+    for (int q = 0; q < NP / 4; ++q) u[q] = u4[q];
+    const bool piv = row == k;
+    const float nf = piv ? 0.f : -(a[0] * rp);
+    if (piv) scale = rp;
+#pragma unroll
+    for (int q = 0; q < NP / 4; ++q) {
+      if (q > 0) a[4 * q - 1] = fmaf(nf, u[q].x, a[4 * q]);
+      a[4 * q] = fmaf(nf, u[q].y, a[4 * q + 1]);
+      a[4 * q + 1] = fmaf(nf, u[q].z, a[4 * q + 2]);
+      a[4 * q + 2] = fmaf(nf, u[q].w, a[4 * q + 3]);
     }
     a[NP - 1] = piv ? 1.f : nf;
+    if (row == k + 1 && k + 1 < N) publish(k + 1);
   }
   for (int k = N; k < NP; ++k) {   // the unused columns go round to the end
     const float t = a[0];
@@ -1201,13 +1234,11 @@ __device__ __noinline__ bool invert(const Team<WPC> tm, const double* M, int N, 
     a[NP - 1] = t;
   }
   if (has) {
-    sc.pinv[row] = m;
 #pragma unroll
     for (int q = 0; q < NP / 4; ++q)
-      __stcg(X4 + q * N + m, make_float4(a[4 * q] * scale, a[4 * q + 1] * scale, a[4 * q + 2] * scale, a[4 * q + 3] * scale));
+      __stcg(X4 + q * N + row, make_float4(a[4 * q] * scale, a[4 * q + 1] * scale, a[4 * q + 2] * scale, a[4 * q + 3] * scale));
   }
   tm.sync();
-  return true;
 }
 
 // r - a x with a rounded to two floats (53 to 48 bits, integer operations) and
@@ -1253,7 +1284,6 @@ __device__ __noinline__ bool solve_inverse(const Team<WPC> tm, const double* M, 
   float4 xr[NP / 4];   // row i of X, for every round
 #pragma unroll
   for (int q = 0; q < NP / 4; ++q) xr[q] = __ldcg(X4 + q * N + i);
-  const int at = sc.pinv[i];
   const double bi = b[i];
   const float wi = isc[i];
   const double* row = M + i * ld;
@@ -1270,7 +1300,7 @@ __device__ __noinline__ bool solve_inverse(const Team<WPC> tm, const double* M, 
     }
     return (s0 + s1) + (s2 + s3);
   };
-  if (has) sc.v[at] = low_float(bi);
+  if (has) sc.v[t] = low_float(bi);
   else if (t < NP) sc.v[t] = 0.f;
   tm.sync();
   const float x0 = apply();
@@ -1307,7 +1337,7 @@ __device__ __noinline__ bool solve_inverse(const Team<WPC> tm, const double* M, 
       if (j < N) r0 = fma(-row[j], x[j], r0);
       rf = low_float(r0 + r1);
     }
-    if (has) sc.v[at] = rf;
+    if (has) sc.v[t] = rf;
     tm.sync();
     const float d = apply();
     xi += double(d);
@@ -1424,6 +1454,7 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
     const double dt = P.dt;
     double t = 0.0;
     bool rejected_last = false;
+    int fell_back = 0;
     double* u1 = w.u;
     double* u2 = w.u + N;
     double* u3 = w.u + 2 * N;
@@ -1439,17 +1470,17 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
       // Refined solves with an FP32 inverse where there is a thread per row (the
       // automatic team sizes up to 128 unknowns); the FP64 matrix stays in
       // shared memory. Beyond that the FP64 LU, or for mixed precision the FP32
-      // LU. Without scratch always the FP64 LU.
-      bool inverse = w.g != nullptr && N <= TS;
-      bool mixed = w.g != nullptr && P.precision == 1 && !inverse;
-      bool ok;
+      // LU. Without scratch always the FP64 LU, and for the rest of a cell that
+      // has fallen back to it twice.
+      bool inverse = w.g != nullptr && N <= TS && fell_back < 2;
+      bool mixed = w.g != nullptr && P.precision == 1 && N > TS;
+      bool ok = true;
       const int ld = m.ld;
       float4* X4 = reinterpret_cast<float4*>(w.g);
       if (inverse) {
         if (tm.tid < N)
           w.inv_isc[tm.tid] = __frcp_rn(fmaf(float(P.rtol), fabsf(low_float(w.y0[tm.tid])), fmaxf(float(P.atol), 1e-30f)));
-        ok = with_padded<WPC>(N, [&](auto np) { return invert<WPC, decltype(np)::value>(tm, w.M, N, ld, w.inv, X4); });
-        if (!ok) inverse = false;
+        with_padded<WPC>(N, [&](auto np) { invert<WPC, decltype(np)::value>(tm, w.M, N, ld, w.inv, X4); });
       }
       // mixed: M goes, transposed, to the team's global copy, and its FP32
       // truncation over M's first half is factorised in shared memory;
@@ -1509,6 +1540,7 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
         // refinement did not converge: redo the stages with the FP64 LU of the kept matrix
         if (tm.tid == 0 && fallbacks) atomicAdd(fallbacks, 1ull);
         if (mixed) restore();
+        if (inverse) ++fell_back;
         mixed = inverse = false;
         ok = lu_factor<WPC, double>(tm, w.M, N, ld, w.invd, w.perm);
       }
