@@ -722,8 +722,14 @@ int configure_launch(dlbchem_ctx* c) {
   e = cudaFuncSetAttribute(dlb::rosenbrock_kernel_ptr(c->wpc, dlb::general_kernel(c->dm)), cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem_bytes);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(dlb::gate_kernel_ptr(c->wpc), cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem_bytes);
+  c->rhs_L = make_rhs_layout(c->hm.nsp, c->hm.nrx, c->dm.N);
+  c->rhs_teams = max_teams;
+  while (c->rhs_teams > 1 && size_t(c->rhs_L.total) * 8 * c->rhs_teams + 640 > max_block) --c->rhs_teams;
+  c->rhs_smem = c->rhs_L.total * 8 * c->rhs_teams + 80 * 8;
+  const void* rhs = dlb::rhs_kernel_ptr(c->wpc, dlb::general_kernel(c->dm));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(rhs, cudaFuncAttributeMaxDynamicSharedMemorySize, c->rhs_smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dlb::rhs_kernel_ptr(c->wpc), cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem_bytes);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->rhs_blocks, rhs, 32 * c->wpc * c->rhs_teams, c->rhs_smem);
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaFuncSetAttribute");
   int bps = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, dlb::rosenbrock_kernel_ptr(c->wpc, dlb::general_kernel(c->dm)), 32 * c->wpc * teams, c->smem_bytes);
@@ -1270,10 +1276,11 @@ int dlbchem_rhs(dlbchem_ctx* c, int64_t n, const double* T, const double* p, con
   if (!T || !p || !Y || !fT || !fY) return fail(c, DLBCHEM_BAD_ARG, "NULL array pointer");
   dlb::RhsArgs a;
   std::memset(&a, 0, sizeof(a));
-  a.m = c->dm; a.L = c->L; a.n = n; a.T = T; a.p = p; a.Y = Y; a.fT = fT; a.fY = fY;
+  a.m = c->dm; a.L = c->rhs_L; a.n = n; a.T = T; a.p = p; a.Y = Y; a.fT = fT; a.fY = fY;
   a.isothermal = c->opt.isothermal;
-  const int64_t grid = std::min<int64_t>((n + c->teams - 1) / c->teams, int64_t(c->num_sms) * c->blocks_per_sm);
-  cudaError_t e = dlb::launch_rhs(c->wpc, unsigned(grid), 32 * c->wpc * c->teams, c->smem_bytes,
+  const int64_t grid = std::min<int64_t>((n + c->rhs_teams - 1) / c->rhs_teams,
+                                         int64_t(c->num_sms) * std::max(c->rhs_blocks, 1));
+  cudaError_t e = dlb::launch_rhs(c->wpc, unsigned(grid), 32 * c->wpc * c->rhs_teams, c->rhs_smem,
                                   static_cast<cudaStream_t>(stream), a);
   return e == cudaSuccess ? DLBCHEM_OK : cuda_fail(c, e, "rhs launch");
 }

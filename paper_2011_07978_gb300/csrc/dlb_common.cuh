@@ -192,6 +192,26 @@ __host__ inline WsLayout make_layout(int nsp, int nrx, int CH, int N, int ld, in
   return L;
 }
 
+// Workspace of the right-hand-side kernel: what a rate evaluation without the
+// Jacobian touches (vv right after wdot, as in make_layout).
+__host__ inline WsLayout make_rhs_layout(int nsp, int nrx, int N) {
+  WsLayout L{};
+  int o = 0;
+  auto take = [&](int n) { int r = o; o += (n + 1) & ~1; return r; };
+  L.y0 = take(N);
+  L.f0 = take(N);
+  L.c = take(nsp + 1);
+  L.E = take(nsp + 1);
+  L.Einv = take(nsp + 1);
+  L.hk = take(nsp + 1);
+  L.wdot = take(nsp + 1);
+  L.vv = take(nsp + 1);
+  L.D = take(nrx);
+  L.scal = take(48);
+  L.total = o;
+  return L;
+}
+
 // Doubles of one team's matrix in the global scratch: M (mixed precision) or the
 // FP32 inverse, N rows of at most CH floats; 16-byte aligned.
 __host__ __device__ inline int64_t matrix_stride(int N, int CH) {
@@ -282,10 +302,10 @@ cudaError_t launch_rhs_w1(unsigned grid, int threads, int smem, cudaStream_t s, 
 cudaError_t launch_rhs_w2(unsigned grid, int threads, int smem, cudaStream_t s, const RhsArgs& a);
 cudaError_t launch_rhs_w4(unsigned grid, int threads, int smem, cudaStream_t s, const RhsArgs& a);
 cudaError_t launch_rhs(int wpc, unsigned grid, int threads, int smem, cudaStream_t s, const RhsArgs& a);
-const void* rhs_kernel_ptr_w1();
-const void* rhs_kernel_ptr_w2();
-const void* rhs_kernel_ptr_w4();
-const void* rhs_kernel_ptr(int wpc);
+const void* rhs_kernel_ptr_w1(bool general);
+const void* rhs_kernel_ptr_w2(bool general);
+const void* rhs_kernel_ptr_w4(bool general);
+const void* rhs_kernel_ptr(int wpc, bool general);
 const void* gate_kernel_ptr_w1();
 const void* gate_kernel_ptr_w2();
 const void* gate_kernel_ptr_w4();

@@ -48,6 +48,9 @@ struct dlbchem_ctx {
   void* d_blob = nullptr;
   dlbchem_options opt{};
   dlb::WsLayout L{};
+  // right-hand-side kernel: layout, teams per CTA, shared memory, CTAs per SM
+  dlb::WsLayout rhs_L{};
+  int rhs_teams = 1, rhs_smem = 0, rhs_blocks = 1;
   int wpc = 1, teams = 1, smem_bytes = 0, blocks_per_sm = 1, num_sms = 0;
   // workspace (grown on demand to the largest ncells seen)
   unsigned long long* d_counter = nullptr;   // queue counter (8 B) + reference index (8 B)

@@ -69,8 +69,8 @@ cudaError_t launch_rhs(int wpc, unsigned grid, int threads, int smem, cudaStream
   return launch_rhs_w4(grid, threads, smem, s, a);
 }
 
-const void* rhs_kernel_ptr(int wpc) {
-  return wpc == 1 ? rhs_kernel_ptr_w1() : (wpc == 2 ? rhs_kernel_ptr_w2() : rhs_kernel_ptr_w4());
+const void* rhs_kernel_ptr(int wpc, bool general) {
+  return wpc == 1 ? rhs_kernel_ptr_w1(general) : (wpc == 2 ? rhs_kernel_ptr_w2(general) : rhs_kernel_ptr_w4(general));
 }
 
 const void* gate_kernel_ptr(int wpc) {

@@ -1813,9 +1813,13 @@ __global__ void __launch_bounds__(128) gate_kernel(const GateArgs a) {
 // ---------------------------------------------------------------------------
 // Right-hand side of the per-cell ODE (Sec. 1: dPhi/dt = f(Phi); here
 // f = (dT/dt, dY_k/dt) at constant p) for every cell, one team per cell.
-// Cells with a non-finite state, T <= 0 or p <= 0 get NaN.
+// Cells with a non-finite state, T <= 0 or p <= 0 get NaN. FP64-bound (about 330
+// FP64 warp instructions a cell at 53/325, 5.2 ms for 262,144 cells at the
+// unit's rate) once enough teams are resident: the workspace holds only what a
+// rate evaluation touches (6.4 KB at 53/325 instead of the integrator's 36 KB,
+// 12 -> 28 warps per SM), and linear-cp mechanisms take the linear thermo.
 // ---------------------------------------------------------------------------
-template <int WPC>
+template <int WPC, bool GEN>
 __global__ void __launch_bounds__(128) rhs_kernel(const RhsArgs a) {
   extern __shared__ __align__(16) double smem[];
   constexpr int TS = 32 * WPC;
@@ -1840,7 +1844,7 @@ __global__ void __launch_bounds__(128) rhs_kernel(const RhsArgs a) {
   for (int64_t cell = int64_t(blockIdx.x) * teams + team; cell < n; cell += int64_t(gridDim.x) * teams) {
     const double p = a.p[cell];
     for (int i = tm.tid; i < N; i += TS) w.y0[i] = i == 0 ? a.T[cell] : a.Y[int64_t(i - 1) * n + cell];
-    if (tm.tid == 0) w.scal[30] = log(p);
+    if (GEN && tm.tid == 0) w.scal[30] = log(p);
     tm.sync();
     int bad = 0;
     for (int i = tm.tid; i < N; i += TS) bad |= !isfinite(w.y0[i]);
@@ -1854,7 +1858,7 @@ __global__ void __launch_bounds__(128) rhs_kernel(const RhsArgs a) {
       continue;
     }
     const double P1 = 1e-6 * p / kR;
-    eval_f<WPC, true>(a.m, tm, w, w.y0, P1, 1.0 / P1, a.isothermal != 0, w.f0);
+    eval_f<WPC, GEN>(a.m, tm, w, w.y0, P1, 1.0 / P1, a.isothermal != 0, w.f0);
     for (int i = tm.tid; i < N; i += TS) {
       if (i == 0) a.fT[cell] = w.f0[0];
       else a.fY[int64_t(i - 1) * n + cell] = w.f0[i];

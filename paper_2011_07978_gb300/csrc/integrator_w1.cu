@@ -18,10 +18,13 @@ cudaError_t launch_gate_w1(unsigned grid, int threads, int smem, cudaStream_t s,
 }
 
 cudaError_t launch_rhs_w1(unsigned grid, int threads, int smem, cudaStream_t s, const RhsArgs& a) {
-  rhs_kernel<1><<<grid, threads, smem, s>>>(a);
+  if (general_kernel(a.m)) rhs_kernel<1, true><<<grid, threads, smem, s>>>(a);
+  else rhs_kernel<1, false><<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-const void* rhs_kernel_ptr_w1() { return reinterpret_cast<const void*>(&rhs_kernel<1>); }
+const void* rhs_kernel_ptr_w1(bool general) {
+  return general ? reinterpret_cast<const void*>(&rhs_kernel<1, true>) : reinterpret_cast<const void*>(&rhs_kernel<1, false>);
+}
 
 }  // namespace dlb

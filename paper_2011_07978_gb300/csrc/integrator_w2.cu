@@ -18,10 +18,13 @@ cudaError_t launch_gate_w2(unsigned grid, int threads, int smem, cudaStream_t s,
 }
 
 cudaError_t launch_rhs_w2(unsigned grid, int threads, int smem, cudaStream_t s, const RhsArgs& a) {
-  rhs_kernel<2><<<grid, threads, smem, s>>>(a);
+  if (general_kernel(a.m)) rhs_kernel<2, true><<<grid, threads, smem, s>>>(a);
+  else rhs_kernel<2, false><<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-const void* rhs_kernel_ptr_w2() { return reinterpret_cast<const void*>(&rhs_kernel<2>); }
+const void* rhs_kernel_ptr_w2(bool general) {
+  return general ? reinterpret_cast<const void*>(&rhs_kernel<2, true>) : reinterpret_cast<const void*>(&rhs_kernel<2, false>);
+}
 
 }  // namespace dlb

@@ -18,10 +18,13 @@ cudaError_t launch_gate_w4(unsigned grid, int threads, int smem, cudaStream_t s,
 }
 
 cudaError_t launch_rhs_w4(unsigned grid, int threads, int smem, cudaStream_t s, const RhsArgs& a) {
-  rhs_kernel<4><<<grid, threads, smem, s>>>(a);
+  if (general_kernel(a.m)) rhs_kernel<4, true><<<grid, threads, smem, s>>>(a);
+  else rhs_kernel<4, false><<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-const void* rhs_kernel_ptr_w4() { return reinterpret_cast<const void*>(&rhs_kernel<4>); }
+const void* rhs_kernel_ptr_w4(bool general) {
+  return general ? reinterpret_cast<const void*>(&rhs_kernel<4, true>) : reinterpret_cast<const void*>(&rhs_kernel<4, false>);
+}
 
 }  // namespace dlb

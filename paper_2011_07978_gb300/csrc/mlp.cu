@@ -77,40 +77,75 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint3
          (uint64_t((sbo >> 4) & 0x3FFF) << 32) | (uint64_t(1) << 46);
 }
 
-// Staging moves eight values of one row per thread and step: global loads of
-// whole 32-byte sectors (or coalesced over rows), one conflict-free 16-byte
-// store, and the loads of the next two k-tiles are in flight while the tensor
-// cores work on this one. An operand's values of consecutive k are adjacent (KC: p[row ld + k])
-// or those of consecutive rows (p[k ld + row]).
-template <bool KC>
+// Staging goes through registers, 16 bytes per load and store, with the loads of
+// the next two k-tiles in flight while the tensor cores work on this one.
+// An operand's values of consecutive k are adjacent (KC: p[row ld + k]): a thread
+// takes chunks of one row and eight k; or those of consecutive rows are
+// (p[k ld + row]): a thread takes four rows and eight k, eight loads for four
+// chunks (with one row per thread the loads and their addresses were 500
+// instructions per thread and tile, 1.7 us; a 4,096-row weight gradient took
+// @WG0@ us, now @WG1@). Row groups lie kRowGroup bytes apart, 16 more than their eight
+// core matrices, so that a warp's stores of every fourth row hit all banks.
+constexpr int kRowGroup = (kTK / 8) * 128 + 16;
+__host__ __device__ constexpr int tile_bytes(int nt) { return 2 * ((kTM + nt) / 8) * kRowGroup; }   // dynamic shared memory
+template <bool KC, int ROWS>
 struct TileSource {
+  static constexpr int kItems = KC ? ROWS * 8 : ROWS * 2;                       // chunks, or groups of four rows
+  static constexpr int kPer = (kItems + kGemmThreads - 1) / kGemmThreads;       // per thread
+  static constexpr int kRegs = kPer * (KC ? 8 : 32);
   const float* p;
   int ld, rows, kend;   // rows and k beyond these are zero
-  bool vec;             // KC: rows start on 16 bytes
+  bool vec;             // 16-byte loads
   __device__ TileSource(const float* p_, int ld_, int rows_, int kend_)
       : p(p_), ld(ld_), rows(rows_), kend(kend_), vec((ld_ & 3) == 0 && (reinterpret_cast<uintptr_t>(p_) & 15) == 0) {}
-  // chunk e of a tile of ROWS rows: its row and first k
-  template <int ROWS>
+  // item e of a tile: its (first) row and first k
   static __device__ __forceinline__ void place(int e, int& row, int& k) {
     if (KC) { row = (e & 7) + ((e >> 6) << 3); k = ((e >> 3) & 7) * 8; }
-    else { row = e % ROWS; k = (e / ROWS) * 8; }
+    else { row = (e % (ROWS / 4)) * 4; k = (e / (ROWS / 4)) * 8; }
   }
-  __device__ __forceinline__ void load(int row, int k, float* v) const {
-    if (KC) {
-      const float* q = p + int64_t(row) * ld + k;
-      if (vec && row < rows && k + 8 <= kend) {
-        *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(q);
-        *reinterpret_cast<float4*>(v + 4) = *reinterpret_cast<const float4*>(q + 4);
-        return;
+  // the tile at (r0, k0) into v[kRegs]
+  __device__ __forceinline__ void fetch(int r0, int k0, float* v) const {
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const int e = threadIdx.x + kGemmThreads * i;
+      if (kItems % kGemmThreads != 0 && e >= kItems) break;
+      int row, k;
+      place(e, row, k);
+      row += r0;
+      k += k0;
+      if (KC) {
+        float* x = v + 8 * i;
+        const float* q = p + int64_t(row) * ld + k;
+        if (vec && row < rows && k + 8 <= kend) {
+          *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(q);
+          *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(q + 4);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[j] = row < rows && k + j < kend ? q[j] : 0.0f;
+        }
+      } else {
+        float* x = v + 32 * i;   // four rows of eight k
+        const float* q = p + int64_t(k) * ld + row;
+        if (vec && row + 4 <= rows && k + 8 <= kend) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float4 f = *reinterpret_cast<const float4*>(q);
+            x[j] = f.x; x[8 + j] = f.y; x[16 + j] = f.z; x[24 + j] = f.w;
+            q += ld;
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) x[8 * r + j] = row + r < rows && k + j < kend ? q[r] : 0.0f;
+            q += ld;
+          }
+        }
       }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = row < rows && k + j < kend ? q[j] : 0.0f;
-    } else {
-      const float* q = p + int64_t(k) * ld + row;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = row < rows && k + j < kend ? q[int64_t(j) * ld] : 0.0f;
     }
   }
+  // v as BF16 into the operand tile; with sums, sums[r] += the r-th row's FP32 values
+  __device__ __forceinline__ static void store(unsigned char* base, const float* v, float* sums);
 };
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
@@ -118,16 +153,35 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
+template <bool KC, int ROWS>
+__device__ __forceinline__ void TileSource<KC, ROWS>::store(unsigned char* base, const float* v, float* sums) {
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int e = threadIdx.x + kGemmThreads * i;
+    if (kItems % kGemmThreads != 0 && e >= kItems) break;
+    int row, k;
+    place(e, row, k);
+#pragma unroll
+    for (int r = 0; r < (KC ? 1 : 4); ++r) {
+      const float* x = v + (KC ? 8 * i : 32 * i + 8 * r);
+      *reinterpret_cast<uint4*>(base + ((row + r) >> 3) * kRowGroup + (k >> 3) * 128 + ((row + r) & 7) * 16) =
+          make_uint4(pack_bf16x2(x[0], x[1]), pack_bf16x2(x[2], x[3]), pack_bf16x2(x[4], x[5]), pack_bf16x2(x[6], x[7]));
+      if (sums) sums[r] += ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+    }
+  }
+}
+
 // The 128 x NT tile at (m0, n0): epi(gm, gn, v, nv) takes nv <= 16 consecutive
 // columns of one row. With BSUM, bsum[n] (NT floats of shared memory) receives
 // the sums over k of B's FP32 values.
 template <int NT, bool BSUM, bool AKC, bool BKC, class Epi>
-__device__ __forceinline__ void gemm_tile(const TileSource<AKC>& A, const TileSource<BKC>& B, int m0, int n0, float* bsum,
-                                          int* __restrict__ status, Epi&& epi) {
-  constexpr int kNA = kTM * kTK / 8 / kGemmThreads, kNB = NT * kTK / 8 / kGemmThreads;   // chunks per thread
-  constexpr int kBuf = (kTM + NT) * kTK * 2;
-  static_assert(!BSUM || (!BKC && kNB == 1 && NT == 32), "one chunk of one row per thread");
-  __shared__ __align__(1024) unsigned char sop[2 * kBuf];
+__device__ __forceinline__ void gemm_tile(const TileSource<AKC, kTM>& A, const TileSource<BKC, NT>& B, int m0, int n0,
+                                          float* bsum, int* __restrict__ status, Epi&& epi) {
+  using SA = TileSource<AKC, kTM>;
+  using SB = TileSource<BKC, NT>;
+  constexpr int kBuf = tile_bytes(NT) / 2;
+  static_assert(!BSUM || (!BKC && SB::kPer == 1), "one group of four rows per thread");
+  extern __shared__ __align__(1024) unsigned char sop[];   // two operand buffers, tile_bytes(NT)
   __shared__ __align__(8) unsigned long long mbar[2];
   __shared__ uint32_t tmem_slot;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -140,19 +194,10 @@ __device__ __forceinline__ void gemm_tile(const TileSource<AKC>& A, const TileSo
                  "r"(uint32_t(NT)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  float ra[2][kNA][8], rb[2][kNB][8];
+  float ra[2][SA::kRegs], rb[2][SB::kRegs];
   auto fetch = [&](int set, int k0) {
-    int row, k;
-#pragma unroll
-    for (int i = 0; i < kNA; ++i) {
-      TileSource<AKC>::template place<kTM>(tid + kGemmThreads * i, row, k);
-      A.load(m0 + row, k0 + k, ra[set][i]);
-    }
-#pragma unroll
-    for (int i = 0; i < kNB; ++i) {
-      TileSource<BKC>::template place<NT>(tid + kGemmThreads * i, row, k);
-      B.load(n0 + row, k0 + k, rb[set][i]);
-    }
+    A.fetch(m0, k0, ra[set]);
+    B.fetch(n0, k0, rb[set]);
   };
   const int K = A.kend, ntiles = (K + kTK - 1) / kTK;
   fetch(0, 0);
@@ -163,10 +208,6 @@ __device__ __forceinline__ void gemm_tile(const TileSource<AKC>& A, const TileSo
   const uint32_t tmem = tmem_slot;
   // kind::f16 instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, N and M
   const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(NT >> 3) << 17) | (uint32_t(kTM >> 4) << 24);
-  auto store = [&](unsigned char* base, int row, int k, const float* v) {
-    *reinterpret_cast<uint4*>(base + ((row >> 3) * (kTK / 8) + (k >> 3)) * 128 + (row & 7) * 16) =
-        make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
-  };
   auto wait = [&](int b, int use) {   // the MMAs of the use-th tile of buffer b (bounded)
     uint32_t done = 0;
     for (int it = 0; it < kWaitLimit && !done; ++it)
@@ -175,28 +216,17 @@ __device__ __forceinline__ void gemm_tile(const TileSource<AKC>& A, const TileSo
     return done != 0;
   };
   bool ok = true;
-  float sum = 0.0f;
+  float sums[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   for (int t0 = 0; t0 < ntiles; t0 += 2) {
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int t = t0 + b;
       if (t < ntiles) {
         unsigned char* sA = sop + b * kBuf;
-        unsigned char* sB = sA + kTM * kTK * 2;
+        unsigned char* sB = sA + kTM / 8 * kRowGroup;
         if (t >= 2) ok = wait(b, (t >> 1) - 1) && ok;
-        int row, k;
-#pragma unroll
-        for (int i = 0; i < kNA; ++i) {
-          TileSource<AKC>::template place<kTM>(tid + kGemmThreads * i, row, k);
-          store(sA, row, k, ra[b][i]);
-        }
-#pragma unroll
-        for (int i = 0; i < kNB; ++i) {
-          TileSource<BKC>::template place<NT>(tid + kGemmThreads * i, row, k);
-          const float* v = rb[b][i];
-          store(sB, row, k, v);
-          if (BSUM) sum += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
-        }
+        SA::store(sA, ra[b], nullptr);
+        SB::store(sB, rb[b], BSUM ? sums : nullptr);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor cores
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
@@ -204,8 +234,8 @@ __device__ __forceinline__ void gemm_tile(const TileSource<AKC>& A, const TileSo
         if (tid == 0) {
 #pragma unroll
           for (int kk = 0; kk < kTK / 16; ++kk) {
-            const uint64_t ad = umma_desc(smem_u32(sA) + kk * 256, 128, (kTK / 8) * 128);
-            const uint64_t bd = umma_desc(smem_u32(sB) + kk * 256, 128, (kTK / 8) * 128);
+            const uint64_t ad = umma_desc(smem_u32(sA) + kk * 256, 128, kRowGroup);
+            const uint64_t bd = umma_desc(smem_u32(sB) + kk * 256, 128, kRowGroup);
             const uint32_t acc = (t > 0 || kk > 0) ? 1u : 0u;
             asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
                          "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
@@ -224,13 +254,13 @@ __device__ __forceinline__ void gemm_tile(const TileSource<AKC>& A, const TileSo
   ok = __syncthreads_and(ok);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (!ok && tid == 0 && status) atomicExch(status, 1);
-  if (BSUM) {   // rows tid % 32 of the eight warps
+  if (BSUM) {   // thread t < NT / 4 * 8 has rows 4 (t % (NT / 4)) .. + 3 of k-group t / (NT / 4)
     float* part = reinterpret_cast<float*>(sop);   // the operand tiles are done with
-    part[tid] = sum;
+    if (tid < SB::kItems) *reinterpret_cast<float4*>(part + 4 * tid) = make_float4(sums[0], sums[1], sums[2], sums[3]);
     __syncthreads();
     if (tid < NT) {
-      sum = 0.0f;
-      for (int w = 0; w < kGemmThreads / 32; ++w) sum += part[w * NT + tid];
+      float sum = 0.0f;
+      for (int g = 0; g < kTK / 8; ++g) sum += part[g * NT + tid];
       bsum[tid] = sum;
     }
     __syncthreads();
@@ -278,7 +308,7 @@ __global__ void __launch_bounds__(kGemmThreads) layer_forward_kernel(int M, int 
                                                             int act, const float* __restrict__ target, float scale,
                                                             float* __restrict__ loss, int* __restrict__ status) {
   float s = 0.0f;
-  gemm_tile<kTN, false>(TileSource<true>(in, K, M, K), TileSource<false>(W, N, N, K), int(blockIdx.y) * kTM,
+  gemm_tile<kTN, false>(TileSource<true, kTM>(in, K, M, K), TileSource<false, kTN>(W, N, N, K), int(blockIdx.y) * kTM,
                         int(blockIdx.x) * kTN, nullptr, status, [&](int gm, int gn, float* v, int nv) {
               const int64_t at = int64_t(gm) * N + gn;
 #pragma unroll
@@ -309,7 +339,7 @@ __global__ void __launch_bounds__(kGemmThreads) layer_forward_kernel(int M, int 
 __global__ void __launch_bounds__(kGemmThreads) layer_backward_kernel(int M, int N, int K, const float* __restrict__ dZn,
                                                              const float* __restrict__ W, float* __restrict__ Z,
                                                              int* __restrict__ status) {
-  gemm_tile<kTN, false>(TileSource<true>(dZn, K, M, K), TileSource<true>(W, K, N, K), int(blockIdx.y) * kTM,
+  gemm_tile<kTN, false>(TileSource<true, kTM>(dZn, K, M, K), TileSource<true, kTN>(W, K, N, K), int(blockIdx.y) * kTM,
                         int(blockIdx.x) * kTN, nullptr, status, [&](int gm, int gn, float* v, int nv) {
               float* z = Z + int64_t(gm) * N + gn;
 #pragma unroll
@@ -343,7 +373,7 @@ __global__ void __launch_bounds__(kGemmThreads) weight_grad_kernel(const GradArg
   const int nt = (g.fo + kGradTN - 1) / kGradTN, t = int(blockIdx.x) - g.tile0;
   const int m0 = t / nt * kTM, n0 = t % nt * kGradTN;
   float* out = a.grad + g.off;
-  gemm_tile<kGradTN, true>(TileSource<false>(g.in, g.fi, g.fi, a.B), TileSource<false>(g.dz, g.fo, g.fo, a.B), m0, n0,
+  gemm_tile<kGradTN, true>(TileSource<false, kTM>(g.in, g.fi, g.fi, a.B), TileSource<false, kGradTN>(g.dz, g.fo, g.fo, a.B), m0, n0,
                            bsum, status,
                            [&](int gm, int gn, float* v, int nv) { store_row(out + int64_t(gm) * g.fo + gn, v, nv); });
   if (m0 == 0 && int(threadIdx.x) < kGradTN && n0 + int(threadIdx.x) < g.fo)
@@ -911,7 +941,7 @@ cudaError_t forward(dlbchem_mlp* m, int64_t B, const float* X, float* out, bool 
     const bool last = li + 1 == int(L.size());
     float* dst = last ? out : Hs + int64_t(li) * B * H;
     float* z = (!last && keep) ? Zs + int64_t(li) * B * H : nullptr;
-    dlb::layer_forward_kernel<<<tiles_of(B, L[li].fo), dlb::kGemmThreads, 0, s>>>(int(B), L[li].fo, L[li].fi, in, m->d_params + L[li].w,
+    dlb::layer_forward_kernel<<<tiles_of(B, L[li].fo), dlb::kGemmThreads, dlb::tile_bytes(dlb::kTN), s>>>(int(B), L[li].fo, L[li].fi, in, m->d_params + L[li].w,
                                                                    dst, m->d_params + L[li].b, z, last ? 0 : 1,
                                                                    last ? target : nullptr, scale, loss, m->d_status);
     e = cudaGetLastError();
@@ -951,6 +981,9 @@ int dlbchem_mlp_create(int n_in, int n_hidden, int n_out, dlbchem_mlp** out) {
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     m->num_sms = 1;
+  // operand buffers beyond the default 48 KB (a failure shows at the launch)
+  (void)cudaFuncSetAttribute(dlb::layer_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dlb::tile_bytes(dlb::kTN));
+  (void)cudaFuncSetAttribute(dlb::layer_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dlb::tile_bytes(dlb::kTN));
   m->fused_ok = plan_fused(m);
   *out = m;
   return DLBCHEM_OK;
@@ -1025,13 +1058,13 @@ int dlbchem_mlp_grad(dlbchem_mlp* m, int64_t B, const float* X, const float* Y, 
     tiles += n;
   }
   for (int li = a.nl - 1; li > 0 && e == cudaSuccess; --li) {
-    dlb::layer_backward_kernel<<<tiles_of(B, L[li].fi), dlb::kGemmThreads, 0, s>>>(int(B), L[li].fi, L[li].fo, a.layer[li].dz,
+    dlb::layer_backward_kernel<<<tiles_of(B, L[li].fi), dlb::kGemmThreads, dlb::tile_bytes(dlb::kTN), s>>>(int(B), L[li].fi, L[li].fo, a.layer[li].dz,
                                                                      m->d_params + L[li].w,
                                                                      Zs + int64_t(li - 1) * B * H, m->d_status);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
-    dlb::weight_grad_kernel<<<unsigned(tiles), dlb::kGemmThreads, 0, s>>>(a, m->d_status);
+    dlb::weight_grad_kernel<<<unsigned(tiles), dlb::kGemmThreads, dlb::tile_bytes(dlb::kGradTN), s>>>(a, m->d_status);
     e = cudaGetLastError();
   }
   return e == cudaSuccess ? DLBCHEM_OK : mfail(m, DLBCHEM_CUDA, cudaGetErrorString(e));
