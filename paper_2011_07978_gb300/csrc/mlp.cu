@@ -57,14 +57,17 @@ __device__ __forceinline__ float dsilu_f(float z) {
 // cores: BF16 operands (FP32 rounded while staged) in shared memory in the
 // canonical K-major layout without swizzle (8 x 8 core matrices of 128 B, the
 // K-groups of a row group contiguous), FP32 accumulator in tensor memory. One
-// CTA of 256 threads computes a tile: every thread stages, one thread issues
-// the MMAs of a k-tile (K = 16 each) and commits them to its buffer's mbarrier
-// (two buffers; a buffer is refilled when its MMAs are done, every wait is
-// bounded), then each warp reads 32 accumulator rows from tensor memory for
-// the epilogue. A wait that gives up sets *status, writes NaN and still frees
-// the tensor memory.
+// CTA computes a tile: eight warps stage k-tiles of 64 into a ring of four
+// buffers, one thread of a ninth issues the MMAs of a k-tile (K = 16 each) as
+// its buffer fills and commits them to the buffer's release, and the eight
+// warps read the accumulator from tensor memory for the epilogue. Waits are on
+// mbarriers and bounded; one that gives up stops the others, sets *status,
+// writes NaN and still frees the tensor memory. (With a CTA barrier per k-tile
+// the staging warps waited for each other and for the issue: 2,070 cycles a
+// k-tile of the weight gradients.)
 constexpr int kTM = 128, kTN = 64, kTK = 64;
-constexpr int kGemmThreads = 256;
+constexpr int kGemmThreads = 256;    // staging and epilogue; a warp of its own issues the MMAs
+constexpr int kGemmStages = 4;       // operand buffers
 constexpr int kWaitLimit = 1 << 24;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
@@ -87,7 +90,7 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint3
 // @WG0@ us, now @WG1@). Row groups lie kRowGroup bytes apart, 16 more than their eight
 // core matrices, so that a warp's stores of every fourth row hit all banks.
 constexpr int kRowGroup = (kTK / 8) * 128 + 16;
-__host__ __device__ constexpr int tile_bytes(int nt) { return 2 * ((kTM + nt) / 8) * kRowGroup; }   // dynamic shared memory
+__host__ __device__ constexpr int tile_bytes(int nt) { return kGemmStages * ((kTM + nt) / 8) * kRowGroup; }   // dynamic shared memory
 template <bool KC, int ROWS>
 struct TileSource {
   static constexpr int kItems = KC ? ROWS * 8 : ROWS * 2;                       // chunks, or groups of four rows
@@ -179,14 +182,18 @@ __device__ __forceinline__ void gemm_tile(const TileSource<AKC, kTM>& A, const T
                                           float* bsum, int* __restrict__ status, Epi&& epi) {
   using SA = TileSource<AKC, kTM>;
   using SB = TileSource<BKC, NT>;
-  constexpr int kBuf = tile_bytes(NT) / 2;
+  constexpr int kBuf = tile_bytes(NT) / kGemmStages;
   static_assert(!BSUM || (!BKC && SB::kPer == 1), "one group of four rows per thread");
-  extern __shared__ __align__(1024) unsigned char sop[];   // two operand buffers, tile_bytes(NT)
-  __shared__ __align__(8) unsigned long long mbar[2];
+  extern __shared__ __align__(1024) unsigned char sop[];   // the ring of operand buffers, tile_bytes(NT)
+  __shared__ __align__(8) unsigned long long full[kGemmStages], empty[kGemmStages], done;
   __shared__ uint32_t tmem_slot;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
-    for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[b])) : "memory");
+    for (int b = 0; b < kGemmStages; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[b])), "r"(kGemmThreads / 32) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[b])) : "memory");
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&done)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -194,63 +201,74 @@ __device__ __forceinline__ void gemm_tile(const TileSource<AKC, kTM>& A, const T
                  "r"(uint32_t(NT)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  const int K = A.kend, ntiles = (K + kTK - 1) / kTK;
   float ra[2][SA::kRegs], rb[2][SB::kRegs];
   auto fetch = [&](int set, int k0) {
     A.fetch(m0, k0, ra[set]);
     B.fetch(n0, k0, rb[set]);
   };
-  const int K = A.kend, ntiles = (K + kTK - 1) / kTK;
-  fetch(0, 0);
-  if (ntiles > 1) fetch(1, kTK);
+  const bool stager = warp < kGemmThreads / 32;
+  if (stager) {
+    fetch(0, 0);
+    if (ntiles > 1) fetch(1, kTK);
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
-  // kind::f16 instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, N and M
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(NT >> 3) << 17) | (uint32_t(kTM >> 4) << 24);
-  auto wait = [&](int b, int use) {   // the MMAs of the use-th tile of buffer b (bounded)
-    uint32_t done = 0;
-    for (int it = 0; it < kWaitLimit && !done; ++it)
+  auto wait = [&](unsigned long long* bar, int use) {   // the use-th phase (bounded)
+    uint32_t ok = 0;
+    for (int it = 0; it < kWaitLimit && !ok; ++it)
       asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                   : "=r"(done) : "r"(smem_u32(&mbar[b])), "r"(uint32_t(use) & 1u) : "memory");
-    return done != 0;
+                   : "=r"(ok) : "r"(smem_u32(bar)), "r"(uint32_t(use) & 1u) : "memory");
+    return ok != 0;
   };
   bool ok = true;
   float sums[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int t0 = 0; t0 < ntiles; t0 += 2) {
+  if (stager) {
+    for (int t0 = 0; t0 < ntiles && ok; t0 += 2) {
 #pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const int t = t0 + b;
-      if (t < ntiles) {
-        unsigned char* sA = sop + b * kBuf;
-        unsigned char* sB = sA + kTM / 8 * kRowGroup;
-        if (t >= 2) ok = wait(b, (t >> 1) - 1) && ok;
-        SA::store(sA, ra[b], nullptr);
-        SB::store(sB, rb[b], BSUM ? sums : nullptr);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor cores
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (tid == 0) {
-#pragma unroll
-          for (int kk = 0; kk < kTK / 16; ++kk) {
-            const uint64_t ad = umma_desc(smem_u32(sA) + kk * 256, 128, kRowGroup);
-            const uint64_t bd = umma_desc(smem_u32(sB) + kk * 256, 128, kRowGroup);
-            const uint32_t acc = (t > 0 || kk > 0) ? 1u : 0u;
-            asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-                         "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
-          }
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_u32(&mbar[b]))
-                       : "memory");
+      for (int b = 0; b < 2; ++b) {
+        const int t = t0 + b, st = t % kGemmStages;
+        if (t < ntiles && ok) {
+          unsigned char* sA = sop + st * kBuf;
+          if (t >= kGemmStages) ok = wait(&empty[st], t / kGemmStages - 1);
+          SA::store(sA, ra[b], nullptr);
+          SB::store(sA + kTM / 8 * kRowGroup, rb[b], BSUM ? sums : nullptr);
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor cores
+          __syncwarp();
+          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[st])) : "memory");
+          if (t + 2 < ntiles) fetch(b, (t + 2) * kTK);
         }
-        if (t + 2 < ntiles) fetch(b, (t + 2) * kTK);
       }
     }
+  } else if (lane == 0) {
+    // kind::f16 instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, N and M
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(NT >> 3) << 17) | (uint32_t(kTM >> 4) << 24);
+    for (int t = 0; t < ntiles; ++t) {
+      const int st = t % kGemmStages;
+      if (!wait(&full[st], t / kGemmStages)) { ok = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sA = smem_u32(sop + st * kBuf), sB = sA + kTM / 8 * kRowGroup;
+#pragma unroll
+      for (int kk = 0; kk < kTK / 16; ++kk) {
+        const uint64_t ad = umma_desc(sA + kk * 256, 128, kRowGroup);
+        const uint64_t bd = umma_desc(sB + kk * 256, 128, kRowGroup);
+        const uint32_t acc = (t > 0 || kk > 0) ? 1u : 0u;
+        asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
+                     "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
+      }
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                       smem_u32(&empty[st]))
+                   : "memory");
+    }
+    // covers every MMA issued, also after a wait that gave up
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&done))
+                 : "memory");
   }
-  // the commit of the last tile covers every MMA before it
-  ok = wait((ntiles - 1) & 1, (ntiles - 1) >> 1) && ok;
+  __syncwarp();   // the issuer's other lanes wait here, not in a poll beside it
+  ok = wait(&done, 0) && ok;
   ok = __syncthreads_and(ok);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (!ok && tid == 0 && status) atomicExch(status, 1);
@@ -267,7 +285,7 @@ __device__ __forceinline__ void gemm_tile(const TileSource<AKC, kTM>& A, const T
   }
   // epilogue: warps w and w + 4 hold rows 32 (w % 4) .. + 31 of the tile, half of the columns each, 16 per load
   const int gm = m0 + 32 * (warp & 3) + lane;
-  for (int c0 = (NT / 2) * (warp >> 2), c1 = c0 + NT / 2; c0 < c1; c0 += 16) {
+  for (int c0 = (NT / 2) * (warp >> 2), c1 = stager ? c0 + NT / 2 : 0; c0 < c1; c0 += 16) {
     uint32_t r[16];
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
@@ -302,7 +320,7 @@ __device__ __forceinline__ void store_row(float* dst, const float* v, int nv) {
 // One layer forward: C = act(in W + bias), the pre-activations to Z if given.
 // With a target (the output layer of a training step) C instead receives the
 // gradient of the MSE, 2 (out - y) scale, and *loss the sum of scale (out - y)^2.
-__global__ void __launch_bounds__(kGemmThreads) layer_forward_kernel(int M, int N, int K, const float* __restrict__ in,
+__global__ void __launch_bounds__(kGemmThreads + 32) layer_forward_kernel(int M, int N, int K, const float* __restrict__ in,
                                                             const float* __restrict__ W, float* __restrict__ C,
                                                             const float* __restrict__ bias, float* __restrict__ Z,
                                                             int act, const float* __restrict__ target, float scale,
@@ -336,7 +354,7 @@ __global__ void __launch_bounds__(kGemmThreads) layer_forward_kernel(int M, int 
 
 // One layer backward: Z <- (dZ_next W^T) silu'(Z), in place (M rows, N = the
 // layer's width, K = the next layer's).
-__global__ void __launch_bounds__(kGemmThreads) layer_backward_kernel(int M, int N, int K, const float* __restrict__ dZn,
+__global__ void __launch_bounds__(kGemmThreads + 32) layer_backward_kernel(int M, int N, int K, const float* __restrict__ dZn,
                                                              const float* __restrict__ W, float* __restrict__ Z,
                                                              int* __restrict__ status) {
   gemm_tile<kTN, false>(TileSource<true, kTM>(dZn, K, M, K), TileSource<true, kTN>(W, K, N, K), int(blockIdx.y) * kTM,
@@ -365,7 +383,7 @@ struct GradArgs {
   float* grad;
   GradLayer layer[8];
 };
-__global__ void __launch_bounds__(kGemmThreads) weight_grad_kernel(const GradArgs a, int* __restrict__ status) {
+__global__ void __launch_bounds__(kGemmThreads + 32) weight_grad_kernel(const GradArgs a, int* __restrict__ status) {
   __shared__ float bsum[kGradTN];
   int l = 0;
   while (l + 1 < a.nl && int(blockIdx.x) >= a.layer[l + 1].tile0) ++l;
@@ -941,7 +959,7 @@ cudaError_t forward(dlbchem_mlp* m, int64_t B, const float* X, float* out, bool 
     const bool last = li + 1 == int(L.size());
     float* dst = last ? out : Hs + int64_t(li) * B * H;
     float* z = (!last && keep) ? Zs + int64_t(li) * B * H : nullptr;
-    dlb::layer_forward_kernel<<<tiles_of(B, L[li].fo), dlb::kGemmThreads, dlb::tile_bytes(dlb::kTN), s>>>(int(B), L[li].fo, L[li].fi, in, m->d_params + L[li].w,
+    dlb::layer_forward_kernel<<<tiles_of(B, L[li].fo), dlb::kGemmThreads + 32, dlb::tile_bytes(dlb::kTN), s>>>(int(B), L[li].fo, L[li].fi, in, m->d_params + L[li].w,
                                                                    dst, m->d_params + L[li].b, z, last ? 0 : 1,
                                                                    last ? target : nullptr, scale, loss, m->d_status);
     e = cudaGetLastError();
@@ -983,6 +1001,7 @@ int dlbchem_mlp_create(int n_in, int n_hidden, int n_out, dlbchem_mlp** out) {
     m->num_sms = 1;
   // operand buffers beyond the default 48 KB (a failure shows at the launch)
   (void)cudaFuncSetAttribute(dlb::layer_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dlb::tile_bytes(dlb::kTN));
+  (void)cudaFuncSetAttribute(dlb::weight_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dlb::tile_bytes(dlb::kGradTN));
   (void)cudaFuncSetAttribute(dlb::layer_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dlb::tile_bytes(dlb::kTN));
   m->fused_ok = plan_fused(m);
   *out = m;
@@ -1058,13 +1077,13 @@ int dlbchem_mlp_grad(dlbchem_mlp* m, int64_t B, const float* X, const float* Y, 
     tiles += n;
   }
   for (int li = a.nl - 1; li > 0 && e == cudaSuccess; --li) {
-    dlb::layer_backward_kernel<<<tiles_of(B, L[li].fi), dlb::kGemmThreads, dlb::tile_bytes(dlb::kTN), s>>>(int(B), L[li].fi, L[li].fo, a.layer[li].dz,
+    dlb::layer_backward_kernel<<<tiles_of(B, L[li].fi), dlb::kGemmThreads + 32, dlb::tile_bytes(dlb::kTN), s>>>(int(B), L[li].fi, L[li].fo, a.layer[li].dz,
                                                                      m->d_params + L[li].w,
                                                                      Zs + int64_t(li - 1) * B * H, m->d_status);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
-    dlb::weight_grad_kernel<<<unsigned(tiles), dlb::kGemmThreads, dlb::tile_bytes(dlb::kGradTN), s>>>(a, m->d_status);
+    dlb::weight_grad_kernel<<<unsigned(tiles), dlb::kGemmThreads + 32, dlb::tile_bytes(dlb::kGradTN), s>>>(a, m->d_status);
     e = cudaGetLastError();
   }
   return e == cudaSuccess ? DLBCHEM_OK : mfail(m, DLBCHEM_CUDA, cudaGetErrorString(e));
