@@ -170,24 +170,41 @@ struct Mix {
   double lnp;                                        // ln p (Pa), for PLOG reactions
 };
 
+// double -> float by truncating the significand (integer operations: the FP64
+// unit does conversions at its own rate). Magnitudes below the float normal
+// range flush to zero; above it, infinity and NaN become infinite or NaN.
+__device__ __forceinline__ float low_float(double v) {
+  const unsigned hi = unsigned(__double2hiint(v)), t = hi & 0x7fffffffu;
+  unsigned f = __funnelshift_l(unsigned(__double2loint(v)), t - 0x38000000u, 3);
+  f = t < 0x38100000u ? 0u : (t >= 0x47f00000u ? 0x7f800000u : f);
+  return __uint_as_float(f | (hi & 0x80000000u));
+}
+// float -> double, exactly, by integer operations: zero or normal finite values
+__device__ __forceinline__ double wide_double(float v) {
+  const unsigned b = __float_as_uint(v), t = b & 0x7fffffffu;
+  return __hiloint2double(int((b & 0x80000000u) | (t ? (t >> 3) + 0x38000000u : 0u)), int(b << 29));
+}
+
 // exp(x) by Tang's table-driven method (P. T. P. Tang, ACM TOMS 15(2), 1989):
-// x = (64 m + j) ln2/64 + r with |r| <= ln2/128, exp(x) = 2^m 2^(j/64) e^r.
-// k = 64 m + j is rounded with the 1.5*2^52 shift, r is reduced with a
-// two-constant Cody-Waite split of ln2/64 (32-bit high part, so k*hi is
-// exact), e^r is its degree-5 Taylor polynomial (remainder < 3.5e-17), and
-// 2^m is added to the exponent field. tab[j] = 2^(j/64) rounded to double.
-// About 10 FP64 operations against ~19 for the library exp; |x| >= 700 and
-// NaN go to the library exp.
+// x = (64 m + j) ln2/64 + r with |r| <= ln2/128 (1 + 0.02), exp(x) = 2^m 2^(j/64)
+// e^r. k = 64 m + j is rounded in FP32 (x to 2^-23 only moves ties), r is reduced
+// with a two-constant Cody-Waite split of ln2/64 (32-bit high part, so k*hi is
+// exact), e^r is its degree-5 Taylor polynomial (remainder < 4e-17) whose
+// two leading coefficients are combined in FP32 (their error times r^4 is
+// below 1.1e-18), and 2^m is added to the exponent field. tab[j] = 2^(j/64) rounded
+// to double. Seven FP64 operations (ten with the rounding and the whole
+// polynomial on the FP64 unit, about 19 for the library exp): the FP64 unit takes
+// one warp instruction per 76 cycles, the integer and FP32 pipes one per
+// cycle beside it. |x| >= 700 and NaN go to the library exp.
 static __device__ __noinline__ double exp_library(double x) { return exp(x); }   // one copy, off the hot path
 __device__ __forceinline__ double exp_tab(double x, const double* __restrict__ tab) {
   if ((__double2hiint(x) & 0x7fffffff) >= 0x4085E000) return exp_library(x);   // |x| >= 700 or NaN (700 = 0x4085E000 00000000)
-  const double kShift = 6755399441055744.0;                 // 1.5 * 2^52
-  const double t = fma(x, 92.33248261689366, kShift);       // x * 64 / ln2, rounded to an integer
-  const int ki = __double2loint(t);
-  const double k = t - kShift;
+  const float t = fmaf(low_float(x), 92.332483f, 12582912.0f);   // x * 64 / ln2, rounded to an integer by 1.5*2^23
+  const int ki = __float_as_int(t) - 0x4B400000;
+  const double k = wide_double(__fsub_rn(t, 12582912.0f));
   double r = fma(-k, 0.010830424696905538, x);              // ln2/64, high 32 bits
   r = fma(-k, -6.563929801064195e-13, r);                   // ln2/64, remainder
-  double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+  double p = wide_double(fmaf(low_float(r), 1.0f / 120.0f, 1.0f / 24.0f));
   p = fma(r, p, 1.0 / 6.0);
   p = fma(r, p, 0.5);
   p = fma(r, p, 1.0);
@@ -1143,16 +1160,6 @@ __device__ __forceinline__ float trunc_to_float(double v) {
   else if (ex - 1023 + 127 <= 0) f = 0u;
   else f = (unsigned(ex - 1023 + 127) << 23) | man;
   return __uint_as_float(sign | f);
-}
-
-// double -> float by truncating the significand (integer operations: the FP64
-// unit does conversions at its own rate). Magnitudes below the float normal
-// range flush to zero; above it, infinity and NaN become infinite or NaN.
-__device__ __forceinline__ float low_float(double v) {
-  const unsigned hi = unsigned(__double2hiint(v)), t = hi & 0x7fffffffu;
-  unsigned f = __funnelshift_l(unsigned(__double2loint(v)), t - 0x38000000u, 3);
-  f = t < 0x38100000u ? 0u : (t >= 0x47f00000u ? 0x7f800000u : f);
-  return __uint_as_float(f | (hi & 0x80000000u));
 }
 
 // ---------------------------------------------------------------------------

@@ -170,22 +170,43 @@ __global__ void radix_hist_kernel(const int64_t* __restrict__ mdev, const uint32
   hist[int64_t(threadIdx.x) * ntiles + blockIdx.x] = h[threadIdx.x];   // digit-major
 }
 
-// Exclusive scan over the digit-major histogram (one block).
-__global__ void radix_scan_kernel(int64_t len, int32_t* __restrict__ hist) {
-  __shared__ int32_t part[kSchedThreads];
-  const int64_t per = (len + blockDim.x - 1) / blockDim.x;
-  const int64_t a = threadIdx.x * per, b = min(len, a + per);
-  int32_t s = 0;
-  for (int64_t j = a; j < b; ++j) s += hist[j];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int32_t acc = 0;
-    for (int t = 0; t < int(blockDim.x); ++t) { const int32_t v = part[t]; part[t] = acc; acc += v; }
+// Exclusive scan over the digit-major histogram (one block of 1,024 threads,
+// coalesced chunks of 4,096 with a running carry: 0.40 -> @SCAN@ ms for the
+// 262,144 counts of as many cells, four times per sort; one contiguous range
+// per thread of 256 read the array a 4 KB stride apart).
+constexpr int kScanThreads = 1024;
+__global__ void __launch_bounds__(kScanThreads) radix_scan_kernel(int64_t len, int32_t* __restrict__ hist) {
+  __shared__ int32_t wsum[kScanThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int32_t carry = 0;
+  for (int64_t base = 0; base < len; base += 4 * kScanThreads) {   // len is a multiple of 256
+    const int64_t at = base + 4 * int64_t(threadIdx.x);
+    int4 v = at < len ? *reinterpret_cast<const int4*>(hist + at) : make_int4(0, 0, 0, 0);
+    const int32_t own = v.x + v.y + v.z + v.w;
+    int32_t incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      int32_t s = wsum[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t u = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += u;
+      }
+      wsum[lane] = s;
+    }
+    __syncthreads();
+    const int32_t before = carry + (warp > 0 ? wsum[warp - 1] : 0) + incl - own;
+    if (at < len)
+      *reinterpret_cast<int4*>(hist + at) = make_int4(before, before + v.x, before + v.x + v.y, before + v.x + v.y + v.z);
+    carry += wsum[kScanThreads / 32 - 1];
+    __syncthreads();   // wsum is rewritten
   }
-  __syncthreads();
-  s = part[threadIdx.x];
-  for (int64_t j = a; j < b; ++j) { const int32_t v = hist[j]; hist[j] = s; s += v; }
 }
 
 __global__ void radix_scatter_kernel(const int64_t* __restrict__ mdev, const uint32_t* __restrict__ kin,
@@ -392,7 +413,7 @@ cudaError_t launch_sort(int64_t n, const int64_t* mdev, uint32_t* keys, int32_t*
   int32_t* vb = list_alt;
   for (int p = 0; p < 4; ++p) {
     radix_hist_kernel<<<ntiles, kSchedThreads, 0, s>>>(mdev, ka, 8 * p, ntiles, hist);
-    radix_scan_kernel<<<1, kSchedThreads, 0, s>>>(int64_t(256) * ntiles, hist);
+    radix_scan_kernel<<<1, kScanThreads, 0, s>>>(int64_t(256) * ntiles, hist);
     radix_scatter_kernel<<<ntiles, kSchedThreads, 0, s>>>(mdev, ka, va, 8 * p, ntiles, hist, kb, vb);
     uint32_t* tk = ka; ka = kb; kb = tk;
     int32_t* tv = va; va = vb; vb = tv;
