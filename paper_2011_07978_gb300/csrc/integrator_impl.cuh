@@ -47,8 +47,16 @@ struct Team {
       asm volatile("bar.sync 2, 64;" ::: "memory");
     }
   }
+  // One-warp teams with values in the lower 16 lanes only (zero above): the
+  // butterflies leave out the exchange of the halves.
+  bool half = false;
   // Sum over the team; every thread receives the bitwise-identical result.
   __device__ __forceinline__ double sum(double x) const {
+    if (WPC == 1 && half) {
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      return __shfl_sync(0xffffffffu, x, 0);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     if (WPC == 1) return x;
@@ -83,7 +91,9 @@ struct Team {
     const bool hi = (lane & 16) != 0;
     double keep = hi ? b : a;
     const double send = hi ? a : b;
-    keep += __shfl_xor_sync(0xffffffffu, send, 16);
+    const double other = __shfl_xor_sync(0xffffffffu, send, 16);
+    if (WPC == 1 && half) keep = hi ? other : keep;
+    else keep += other;
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
     a = __shfl_sync(0xffffffffu, keep, 0);
@@ -1561,19 +1571,26 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
         acc = fma(r, r, acc);
         w.ys[i] = yn;
       }
-      const double err2 = tm.sum(acc) * iN;
-      // one warp takes the square roots (60 FP64 instructions) for the team;
-      // 0.9 errn^(-1/4) as rsqrt(sqrt(errn)): within 2 ulp of pow
-      if (tm.warp == 0) {
-        double errn = sqrt(err2);
-        if (!ok) errn = nan("");
-        const double fac = isfinite(errn) ? 0.9 * rsqrt(sqrt(errn)) : 0.2;
-        if (tm.lane == 0) { w.scal[26] = errn; w.scal[27] = fac; }
+      const double err2 = tm.sum(acc) * iN;   // the error norm squared
+      // 0.9 errn^(-1/4) = 0.9 err2^(-1/8): the FP32 estimate y and one
+      // third-order correction, with e = 1 - err2 y^8 (of order 1e-6)
+      // y (1 - e)^(-1/8) = y (1 + e/8 + 9/128 e^2 + ...). Seven FP64 operations;
+      // two square roots and a reciprocal one were 45, a tenth of a step at 11
+      // unknowns. Outside [1e-7, 1e6] the factor is one of its limits.
+      const float ef = low_float(err2);
+      double fac;
+      if (ef > 1e-7f && ef < 1e6f) {
+        const double y = wide_double(exp2f(-0.125f * __log2f(ef)));
+        const double y2 = y * y, y4 = y2 * y2;
+        const double e = fma(-err2, y4 * y4, 1.0);
+        fac = 0.9 * fma(y * e, fma(e, 9.0 / 128.0, 0.125), y);
+      } else {
+        fac = err2 < 1.0 ? 5.0 : 0.2;   // NaN too
       }
-      tm.sync();
-      const double errn = w.scal[26];
-      double fac = fmax(0.2, w.scal[27]);
-      if (errn <= 1.0) {
+      fac = fmax(0.2, fac);
+      const bool accept = ok && err2 <= 1.0;
+      if (!ok) fac = 0.2;
+      if (accept) {
         fac = fmin(5.0, fac);
         if (rejected_last) fac = fmin(fac, 1.0);
         t = (t + h >= dt) ? dt : t + h;
@@ -1614,6 +1631,7 @@ __global__ void __launch_bounds__(128, WPC == 1 ? 4 : (WPC == 2 ? 3 : 2)) rosenb
   tm.lane = threadIdx.x & 31;
   tm.bar_id = 1 + team;
   tm.parity = 0;
+  tm.half = a.m.N <= 16;
   double* tab = smem + size_t(teams) * a.L.total;
   for (int j = threadIdx.x; j < 64; j += blockDim.x) tab[j] = a.m.exptab[j];
   for (int j = threadIdx.x; j < 16; j += blockDim.x) tab[64 + j] = double(j - 8);
@@ -1838,6 +1856,7 @@ __global__ void __launch_bounds__(128) rhs_kernel(const RhsArgs a) {
   tm.lane = threadIdx.x & 31;
   tm.bar_id = 1 + team;
   tm.parity = 0;
+  tm.half = a.m.N <= 16;
   double* tab = smem + size_t(teams) * a.L.total;
   for (int j = threadIdx.x; j < 64; j += blockDim.x) tab[j] = a.m.exptab[j];
   for (int j = threadIdx.x; j < 16; j += blockDim.x) tab[64 + j] = double(j - 8);
