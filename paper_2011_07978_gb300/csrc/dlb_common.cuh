@@ -121,7 +121,7 @@ struct IntegParams {
 struct WsLayout {
   int M, y0, f0, ys, fs, u, c, E, Einv, hk, wdot, vv, dwdT, uu, invd, q, dqdT, dlt, D, scal, perm;
   int M32, invd32, perm32, rr, dx, isc;   // mixed precision with more unknowns than threads only (else 0)
-  int w32, v, xf, invs, rows;             // refined solves with the FP32 inverse
+  int w32, v, xf, xs, invs, rows;         // refined solves with the FP32 inverse
   int total;  // doubles per team (int and float arrays are counted in doubles)
 };
 
@@ -154,12 +154,13 @@ __host__ inline WsLayout make_layout(int nsp, int nrx, int CH, int N, int ld, in
   // refined solves: weights and right-hand side over the Jacobian-only arrays
   // dwdT .. dlt (dead from the assembly of one step to the next), published
   // rows (dead during the rate evaluations too) behind them up to scal
-  L.w32 = L.v = L.xf = L.invs = L.rows = 0;
+  L.w32 = L.v = L.xf = L.xs = L.invs = L.rows = 0;
   if (N <= CH) {
     auto vectors = [&](auto&& take2) {
       L.w32 = take2((N + 1) / 2);
       L.v = take2(CH / 2);
       L.xf = take2((N + 1) / 2);
+      L.xs = take2(N <= 12 && CH == 32 ? 6 * N : 0);   // 12 x N floats
       L.invs = take2(1);
       L.rows = take2(CH);
     };

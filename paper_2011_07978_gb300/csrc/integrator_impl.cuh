@@ -152,6 +152,7 @@ struct WS {
   double *rr, *dx, *isc;
   InvScratch inv;         // refined solves with the FP32 inverse
   float* inv_isc;
+  float4* xs;             // the FP32 inverse of up to kSharedX unknowns
   const double* exptab;   // 64 entries of 2^(j/64), shared by the CTA
   const double* nutab;    // nutab[j] = j - 8: stoichiometric coefficients by their 4-bit code
   double* g;              // this team's global scratch (L2-resident): the FP32 inverse, or mixed
@@ -171,6 +172,7 @@ __device__ __forceinline__ WS carve(double* base, const WsLayout& L) {
   w.inv = InvScratch{reinterpret_cast<float*>(base + L.rows), reinterpret_cast<float*>(base + L.invs),
                      reinterpret_cast<float*>(base + L.v), reinterpret_cast<float*>(base + L.xf)};
   w.inv_isc = reinterpret_cast<float*>(base + L.w32);
+  w.xs = reinterpret_cast<float4*>(base + L.xs);
   return w;
 }
 
@@ -1202,9 +1204,20 @@ __device__ __forceinline__ float trunc_to_float(double v) {
 // preconditioner: on 27,000 steps over the three mechanisms and all classes of
 // states both the pivoted and this inverse took two rounds on every one. Where
 // a pivot is so small that the refinement does not converge, the FP64 LU
-// (partial pivoting) takes the step. X goes to a global per-team scratch (L2),
-// four columns per 16 bytes: X4[q N + row].
+// (partial pivoting) takes the step. X is stored four columns per 16 bytes:
+// X4[q N + row].
 // ---------------------------------------------------------------------------
+// X of up to 12 unknowns lies in shared memory (0.5 KB; the four reads of a step
+// are 3 of 84 kcycles from L2), larger ones in the global scratch.
+constexpr int kSharedX = 12;
+template <int NP>
+__device__ __forceinline__ void put_x(float4* p, float4 v) {
+  if (NP <= kSharedX) *p = v;
+  else __stcg(p, v);
+}
+template <int NP>
+__device__ __forceinline__ float4 get_x(const float4* p) { return NP <= kSharedX ? *p : __ldcg(p); }
+
 template <int WPC, int NP>
 __device__ __noinline__ void invert(const Team<WPC> tm, const double* M, int N, int ld, const InvScratch sc, float4* X4) {
   const int row = tm.tid;
@@ -1228,18 +1241,22 @@ __device__ __noinline__ void invert(const Team<WPC> tm, const double* M, int N, 
     tm.sync();   // row k is there, and row k - 1's buffer is no longer read
     const float4* u4 = reinterpret_cast<const float4*>(sc.rows + (k & 1) * NP);
     const float rp = invs[k & 1];
-    float4 u[NP / 4];
+    // the whole row at once where the registers allow it
+    constexpr int kAhead = NP <= 64 ? NP / 4 : 4;
+    float4 u[kAhead];
 #pragma unroll
-    for (int q = 0; q < NP / 4; ++q) u[q] = u4[q];
+    for (int q = 0; q < kAhead; ++q) u[q] = u4[q];
     const bool piv = row == k;
     const float nf = piv ? 0.f : -(a[0] * rp);
     if (piv) scale = rp;
 #pragma unroll
     for (int q = 0; q < NP / 4; ++q) {
-      if (q > 0) a[4 * q - 1] = fmaf(nf, u[q].x, a[4 * q]);
-      a[4 * q] = fmaf(nf, u[q].y, a[4 * q + 1]);
-      a[4 * q + 1] = fmaf(nf, u[q].z, a[4 * q + 2]);
-      a[4 * q + 2] = fmaf(nf, u[q].w, a[4 * q + 3]);
+      const float4 x = u[q % kAhead];
+      if (q + kAhead < NP / 4) u[q % kAhead] = u4[q + kAhead];
+      if (q > 0) a[4 * q - 1] = fmaf(nf, x.x, a[4 * q]);
+      a[4 * q] = fmaf(nf, x.y, a[4 * q + 1]);
+      a[4 * q + 1] = fmaf(nf, x.z, a[4 * q + 2]);
+      a[4 * q + 2] = fmaf(nf, x.w, a[4 * q + 3]);
     }
     a[NP - 1] = piv ? 1.f : nf;
     if (row == k + 1 && k + 1 < N) publish(k + 1);
@@ -1253,7 +1270,7 @@ __device__ __noinline__ void invert(const Team<WPC> tm, const double* M, int N, 
   if (has) {
 #pragma unroll
     for (int q = 0; q < NP / 4; ++q)
-      __stcg(X4 + q * N + row, make_float4(a[4 * q] * scale, a[4 * q + 1] * scale, a[4 * q + 2] * scale, a[4 * q + 3] * scale));
+      put_x<NP>(X4 + q * N + row, make_float4(a[4 * q] * scale, a[4 * q + 1] * scale, a[4 * q + 2] * scale, a[4 * q + 3] * scale));
   }
   tm.sync();
 }
@@ -1300,7 +1317,7 @@ __device__ __noinline__ bool solve_inverse(const Team<WPC> tm, const double* M, 
   const int i = min(t, N - 1);
   float4 xr[NP / 4];   // row i of X, for every round
 #pragma unroll
-  for (int q = 0; q < NP / 4; ++q) xr[q] = __ldcg(X4 + q * N + i);
+  for (int q = 0; q < NP / 4; ++q) xr[q] = get_x<NP>(X4 + q * N + i);
   const double bi = b[i];
   const float wi = isc[i];
   const double* row = M + i * ld;
@@ -1493,7 +1510,7 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
       bool mixed = w.g != nullptr && P.precision == 1 && N > TS;
       bool ok = true;
       const int ld = m.ld;
-      float4* X4 = reinterpret_cast<float4*>(w.g);
+      float4* X4 = WPC == 1 && N <= kSharedX ? w.xs : reinterpret_cast<float4*>(w.g);
       if (inverse) {
         if (tm.tid < N)
           w.inv_isc[tm.tid] = __frcp_rn(fmaf(float(P.rtol), fabsf(low_float(w.y0[tm.tid])), fmaxf(float(P.atol), 1e-30f)));
