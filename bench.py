@@ -278,9 +278,9 @@ def mlp_forward_rate(dlbchem, dev, stream, n):
     return {"cells": n, "ms": ms, "achieved_tflops": tf, "peak_bf16_tflops": peak, "frac": tf / peak,
             "peak_source": "MEASURED_PEAKS.json bf16_tflops" if os.path.exists(peaks) else "fallback 1.9 PFLOP/s",
             "kernel": ("mlp_fused_forward_kernel (whole network per 128 rows; tcgen05.mma kind::f16, TMEM "
-                       "accumulator, weights by cp.async.bulk)") if fused else "gemm_tc_kernel per layer",
+                       "accumulator, weights by cp.async.bulk)") if fused else "layer_forward_kernel per layer",
             "layered_ms": ms_layered,
-            "layered_kernel": "gemm_tc_kernel per layer (FP32 activations in HBM)"}
+            "layered_kernel": "layer_forward_kernel per layer (FP32 activations in HBM)"}
 
 
 def fp64_probe(dlbchem, dev, stream):
