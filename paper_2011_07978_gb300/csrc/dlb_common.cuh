@@ -117,6 +117,9 @@ struct IntegParams {
   int32_t precision, reserved;   // precision 1: FP32 LU + FP64 refinement
 };
 
+// One-warp teams keep the FP32 inverse of up to this many unknowns in shared memory.
+constexpr int kSharedX = 12;
+
 // Offsets (in doubles) of one team's workspace inside dynamic shared memory.
 struct WsLayout {
   int M, y0, f0, ys, fs, u, c, E, Einv, hk, wdot, vv, dwdT, uu, invd, q, dqdT, dlt, D, scal, perm;
@@ -160,7 +163,7 @@ __host__ inline WsLayout make_layout(int nsp, int nrx, int CH, int N, int ld, in
       L.w32 = take2((N + 1) / 2);
       L.v = take2(CH / 2);
       L.xf = take2((N + 1) / 2);
-      L.xs = take2(N <= 12 && CH == 32 ? 6 * N : 0);   // 12 x N floats
+      L.xs = take2(N <= kSharedX && CH == 32 ? kSharedX * N / 2 : 0);   // kSharedX x N floats
       L.invs = take2(1);
       L.rows = take2(CH);
     };

@@ -2,15 +2,16 @@
 //
 // Paper (arXiv 2011.07978) Sec. 1 / Sec. 2.1: every cell integrates its own
 // stiff ODE dPhi/dt = f(Phi) over the flow step dt; Sec. 2.2 stage 3 is this
-// solve. One team of threads (one warp, or four warps for mechanisms with
-// more than 64 unknowns) owns one cell at a time and keeps the whole cell in
-// shared memory: the dense iteration matrix M = I/(h gamma) - J, the stage
-// vectors and the per-species and per-reaction work arrays. Lanes split
-// species, reactions, matrix entries and rows; FP64 is the bottleneck on
-// GB300 (two FP64 FMA lanes per clock per SM, a warp instruction costs the
-// same whatever its active lanes), so every phase is laid out to keep all 32
-// lanes of a warp busy: flattened trailing updates in the LU, conflict-free
-// rounds of 32 for the sparse scatters.
+// solve. One team of threads (one, two or four warps) owns one cell at a time
+// and keeps the whole cell in shared memory: the dense iteration matrix M =
+// I/(h gamma) - J, the stage vectors and the per-species and per-reaction work
+// arrays. Lanes split species, reactions, matrix entries and rows. FP64 is the
+// bottleneck on GB300 (the unit takes one warp instruction per 76 cycles and SM
+// sub-partition, the same whatever its active lanes, and a dependent one waits
+// 64), so FP64 phases keep the lanes of a warp busy (conflict-free rounds of 32
+// for the sparse scatters), and what needs no FP64 result is off that unit:
+// the linear solves are preconditioned by an FP32 inverse, conversions and
+// range reductions are integer work.
 //
 // Every reduction runs in a fixed order, so a cell's result does not depend
 // on which team, CTA or launch integrates it (plain and queued schedules
@@ -1207,9 +1208,8 @@ __device__ __forceinline__ float trunc_to_float(double v) {
 // (partial pivoting) takes the step. X is stored four columns per 16 bytes:
 // X4[q N + row].
 // ---------------------------------------------------------------------------
-// X of up to 12 unknowns lies in shared memory (0.5 KB; the four reads of a step
+// X of up to kSharedX unknowns lies in shared memory (0.5 KB; the four reads of a step
 // are 3 of 84 kcycles from L2), larger ones in the global scratch.
-constexpr int kSharedX = 12;
 template <int NP>
 __device__ __forceinline__ void put_x(float4* p, float4 v) {
   if (NP <= kSharedX) *p = v;
@@ -1506,11 +1506,12 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
       // shared memory. Beyond that the FP64 LU, or for mixed precision the FP32
       // LU. Without scratch always the FP64 LU, and for the rest of a cell that
       // has fallen back to it twice.
-      bool inverse = w.g != nullptr && N <= TS && fell_back < 2;
+      const bool shared_x = WPC == 1 && N <= kSharedX;
+      bool inverse = (shared_x || w.g != nullptr) && N <= TS && fell_back < 2;
       bool mixed = w.g != nullptr && P.precision == 1 && N > TS;
       bool ok = true;
       const int ld = m.ld;
-      float4* X4 = WPC == 1 && N <= kSharedX ? w.xs : reinterpret_cast<float4*>(w.g);
+      float4* X4 = shared_x ? w.xs : reinterpret_cast<float4*>(w.g);
       if (inverse) {
         if (tm.tid < N)
           w.inv_isc[tm.tid] = __frcp_rn(fmaf(float(P.rtol), fabsf(low_float(w.y0[tm.tid])), fmaxf(float(P.atol), 1e-30f)));
