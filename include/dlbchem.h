@@ -103,8 +103,8 @@ typedef struct dlbchem_options {
                            above with FP32 LU factors) stops when the estimated remaining error
                            is below 1e-6 of the error weights, at most 3 rounds, the step redone
                            with the FP64 LU if they do not converge. State, rates, error norm
-                           and step control are FP64 in both. Fixed at create, which (beyond 12
-                           unknowns) allocates one matrix per resident team (SMs x CTAs per SM x teams; 22 MB at 54
+                           and step control are FP64 in both. Fixed at create, which allocates
+                           one matrix per resident team (SMs x CTAs per SM x teams; 22 MB at 54
                            unknowns on 152 SMs); if that fails, precision 0 runs the FP64 LU
                            throughout and precision 1 returns OOM. Mixed-precision contexts always
                            launch persistent teams (the plain schedule keeps index order). */

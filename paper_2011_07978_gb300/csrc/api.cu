@@ -1004,8 +1004,7 @@ int dlbchem_create(const char* mech_path, const dlbchem_options* opt, dlbchem_ct
   // so that callers who reserve their memory after creating the context
   // find it in place (a failure here is retried by the first static call)
   (void)dlb::static_scratch_prepare(c->device);
-  const bool shared_x = c->wpc == 1 && c->dm.N <= dlb::kSharedX;   // needs no global matrix
-  if ((o.precision == 1 || c->dm.N <= 32 * c->wpc) && !shared_x) {
+  if (o.precision == 1 || c->dm.N <= 32 * c->wpc) {
     const size_t slots = size_t(c->num_sms) * c->blocks_per_sm;
     const std::vector<unsigned> zero(slots, 0u);
     if (cudaMalloc(&c->d_m64, slots * c->teams * dlb::matrix_stride(c->dm.N, c->dm.CH) * sizeof(double)) != cudaSuccess ||

@@ -1506,12 +1506,11 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
       // shared memory. Beyond that the FP64 LU, or for mixed precision the FP32
       // LU. Without scratch always the FP64 LU, and for the rest of a cell that
       // has fallen back to it twice.
-      const bool shared_x = WPC == 1 && N <= kSharedX;
-      bool inverse = (shared_x || w.g != nullptr) && N <= TS && fell_back < 2;
+      bool inverse = w.g != nullptr && N <= TS && fell_back < 2;
       bool mixed = w.g != nullptr && P.precision == 1 && N > TS;
       bool ok = true;
       const int ld = m.ld;
-      float4* X4 = shared_x ? w.xs : reinterpret_cast<float4*>(w.g);
+      float4* X4 = WPC == 1 && N <= kSharedX ? w.xs : reinterpret_cast<float4*>(w.g);
       if (inverse) {
         if (tm.tid < N)
           w.inv_isc[tm.tid] = __frcp_rn(fmaf(float(P.rtol), fabsf(low_float(w.y0[tm.tid])), fmaxf(float(P.atol), 1e-30f)));
