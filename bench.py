@@ -50,7 +50,7 @@ FP64_PEAK_TFLOPS = 152 * 2.07e9 * 2 * 2 / 1e12
 # read, 0 written, 912 cells integrated on the 8,192-cell bimodal field with
 # bucket mapping), scaled by the cells the benchmark's launch integrates; None
 # whenever the kernel has changed since the capture.
-INTEGRATOR_TRAFFIC_BYTES_PER_CELL = 4040960 / 912
+INTEGRATOR_TRAFFIC_BYTES_PER_CELL = 4520960 / 912
 N_F = 3   # function evaluations per Rosenbrock step (stage 4 reuses stage 3's)
 PAPER_CONTEXT = ("paper (DLBFoam, arXiv 2011.07978): load balancing + reference mapping speed the CPU "
                  "chemistry step up by about 10x (Spray A, 256 MPI ranks on 2x64-core AMD EPYC Rome nodes, "
