@@ -610,10 +610,9 @@ bool build_tables(const dlb::HostMech& hm, int wpc, std::vector<unsigned char>& 
   std::vector<double> nasa(size_t(2) * kNasaStride * std::max(nsp, 1) + std::max(nsp, 1), 0.0);
   int nplog = 0;
   for (const auto& x : hm.rx) nplog += x.plog.empty() ? 0 : 1;
-  // the general instantiation (PLOG or NASA-7) and the gate and right-hand-side
-  // kernels always read NASA-7 tables: a linear-cp mechanism gets its exact
-  // NASA-7 form (a1 = a/R, a2 = b/R, a6 and a7 from hf and s0 at T0, both
-  // ranges alike)
+  // the general instantiations (PLOG or NASA-7) and the gate kernel always read
+  // NASA-7 tables: a linear-cp mechanism gets its exact NASA-7 form (a1 = a/R,
+  // a2 = b/R, a6 and a7 from hf and s0 at T0, both ranges alike)
   std::vector<double> lin_nasa;
   const std::vector<double>* src = &hm.nasa;
   if (hm.nasa.empty()) {

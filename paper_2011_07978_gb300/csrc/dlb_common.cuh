@@ -77,9 +77,9 @@ struct DevMech {
   int nplog;              // PLOG reactions
   int nasa_file;          // the mechanism's thermo is NASA-7 (else cp = a + b T)
   // NASA-7 thermo for every mechanism (a linear-cp one in its exact NASA-7
-  // form), read by the general instantiation and the gate and right-hand-side
-  // kernels: per species and range (low, high) kNasaStride folded coefficients,
-  // then each species' Tmid
+  // form), read by the general instantiations and the gate kernel: per species
+  // and range (low, high) kNasaStride folded coefficients, then each species'
+  // Tmid
   const double* nasa;
   const double* nasa_tmid;
   const int32_t* eff_sp;

@@ -1185,12 +1185,13 @@ __device__ __forceinline__ float trunc_to_float(double v) {
 // the residual against the FP64 matrix. An inverse and not an LU because a
 // triangular sweep is a chain of N columns (8.4 kcycles for 54 unknowns, 12
 // sweeps per step) and a product with X is none.
-// Measured per step, FP64 LU and solves before: 53 species, two warps per
-// cell, 224 -> 149 us alone on an SM, 309 -> 241 us with six cells (FP64 warp
-// instructions 5,040 -> about 3,300); 100 species, four warps, 540 -> 332 us
-// with two cells; 10 species, one warp, 51 -> 43 us. The error against a
-// 64-bit integration is the same (1.3e-14 and 1.4e-14 relative in Y on 4,001
-// cells of 53 species, 1.1e-13 and 1.1e-13 on 400 of 100).
+// Measured per step, FP64 LU and sweeps before, this and the shorter rounds and
+// exponentials now: 53 species, two warps per cell, 224 -> 126 us alone on an SM,
+// 309 -> 196 us with six cells (FP64 warp instructions 5,040 -> 2,600); 100
+// species, four warps, 540 -> 260 us with two cells; 10 species, one warp, 51 ->
+// 41 us. The inverse alone brought 309 -> 241, 540 -> 332 and 51 -> 43 us. The
+// error against a 64-bit integration is the same: before and now 3.2e-14 relative
+// in Y on 4,001 cells of 53 species, 1.8e-13 on 400 of 100.
 //
 // Gauss-Jordan elimination in registers: thread i holds row i. Per column k the
 // owner of row k has published it (double-buffered), one barrier, and every
