@@ -27,12 +27,12 @@
 
 namespace dlb {
 
+// The threads of a team and their barrier: values only, so functions that are
+// not inlined take it by value (by reference it would live in local memory).
 template <int WPC>
-struct Team {
+struct TeamThreads {
   static constexpr int TS = 32 * WPC;
   int tid, warp, lane, bar_id;
-  double* red;          // 2*WPC doubles of cross-warp reduction scratch
-  mutable int parity;
 
   __device__ __forceinline__ void sync() const {
     // Immediate barrier ids: a register id makes ptxas reserve all 16 named
@@ -48,6 +48,37 @@ struct Team {
       asm volatile("bar.sync 2, 64;" ::: "memory");
     }
   }
+  // Team maxima of two unsigned keys (every thread receives both), through
+  // WPC doubles at buf. Nothing orders the reads of buf after the barrier: two
+  // calls in a row need different slots.
+  __device__ __forceinline__ void umax2(unsigned& a, unsigned& b, double* buf) const {
+    a = __reduce_max_sync(0xffffffffu, a);
+    b = __reduce_max_sync(0xffffffffu, b);
+    if (WPC == 1) return;
+    unsigned* ub = reinterpret_cast<unsigned*>(buf);
+    if (lane == 0) { ub[2 * warp] = a; ub[2 * warp + 1] = b; }
+    sync();
+#pragma unroll
+    for (int w = 0; w < WPC; ++w) { a = max(a, ub[2 * w]); b = max(b, ub[2 * w + 1]); }
+  }
+};
+
+// A team with its reductions. They alternate between two sets of slots, as one
+// barrier orders the writes of a reduction before its reads and nothing orders
+// these reads before the next one's writes; which set is next is state of the
+// team, so it is not copied: a copy that reduces leaves the original to write
+// slots that a slower warp still reads.
+template <int WPC>
+struct Team : TeamThreads<WPC> {
+  using TeamThreads<WPC>::lane;
+  using TeamThreads<WPC>::warp;
+  using TeamThreads<WPC>::sync;
+  double* red;          // 2*WPC doubles of cross-warp reduction scratch
+  mutable int parity;
+  Team() = default;
+  Team(const Team&) = delete;
+  Team& operator=(const Team&) = delete;
+
   // One-warp teams with values in the lower 16 lanes only (zero above): the
   // butterflies leave out the exchange of the halves.
   bool half = false;
@@ -111,16 +142,9 @@ struct Team {
   }
   // Team maxima of two unsigned keys (every thread receives both).
   __device__ __forceinline__ void umax2(unsigned& a, unsigned& b) const {
-    a = __reduce_max_sync(0xffffffffu, a);
-    b = __reduce_max_sync(0xffffffffu, b);
-    if (WPC == 1) return;
     double* buf = red + parity * WPC;
     parity ^= 1;
-    unsigned* ub = reinterpret_cast<unsigned*>(buf);
-    if (lane == 0) { ub[2 * warp] = a; ub[2 * warp + 1] = b; }
-    sync();
-#pragma unroll
-    for (int w = 0; w < WPC; ++w) { a = max(a, ub[2 * w]); b = max(b, ub[2 * w + 1]); }
+    TeamThreads<WPC>::umax2(a, b, buf);
   }
   __device__ __forceinline__ int any(int x) const {
     x = __any_sync(0xffffffffu, x);
@@ -142,6 +166,7 @@ struct InvScratch {
   float* invs;      // [2] reciprocals of their pivots
   float* v;         // [NP] right-hand side
   float* xf;        // [N] first solution
+  double* keys;     // [2][WPC] convergence maxima, slots of their own
 };
 
 struct WS {
@@ -171,7 +196,7 @@ __device__ __forceinline__ WS carve(double* base, const WsLayout& L) {
   w.perm32 = reinterpret_cast<int*>(base + L.perm32);
   w.rr = base + L.rr; w.dx = base + L.dx; w.isc = base + L.isc;
   w.inv = InvScratch{reinterpret_cast<float*>(base + L.rows), reinterpret_cast<float*>(base + L.invs),
-                     reinterpret_cast<float*>(base + L.v), reinterpret_cast<float*>(base + L.xf)};
+                     reinterpret_cast<float*>(base + L.v), reinterpret_cast<float*>(base + L.xf), base + L.scal + 16};
   w.inv_isc = reinterpret_cast<float*>(base + L.w32);
   w.xs = reinterpret_cast<float4*>(base + L.xs);
   return w;
@@ -1220,7 +1245,7 @@ template <int NP>
 __device__ __forceinline__ float4 get_x(const float4* p) { return NP <= kSharedX ? *p : __ldcg(p); }
 
 template <int WPC, int NP>
-__device__ __noinline__ void invert(const Team<WPC> tm, const double* M, int N, int ld, const InvScratch sc, float4* X4) {
+__device__ __noinline__ void invert(const TeamThreads<WPC> tm, const double* M, int N, int ld, const InvScratch sc, float4* X4) {
   const int row = tm.tid;
   const bool has = row < N;
   float scale = 0.f;
@@ -1310,7 +1335,7 @@ __device__ __forceinline__ void sub_product(float& s, float& low, double a, floa
 //    that; at most three rounds.
 // Returns false if it did not converge (the caller then takes the FP64 LU).
 template <int WPC, int NP>
-__device__ __noinline__ bool solve_inverse(const Team<WPC> tm, const double* M, int N, int ld, const InvScratch sc,
+__device__ __noinline__ bool solve_inverse(const TeamThreads<WPC> tm, const double* M, int N, int ld, const InvScratch sc,
                                            const float4* X4, const double* b, double* x, const float* isc, bool tight) {
   constexpr bool kPairs = NP > 32;   // below, the FP64 residual is short (0.4 kcycles less per solve at 11 unknowns)
   const int t = tm.tid;
@@ -1381,7 +1406,7 @@ __device__ __noinline__ bool solve_inverse(const Team<WPC> tm, const double* M, 
     // maxima of values that are non-negative, infinite or NaN, by bit pattern
     unsigned ud = has ? __float_as_uint(fabsf(d) * wi) : 0u;
     unsigned ux = has ? __float_as_uint(fabsf(low_float(xi)) * wi) : 0u;
-    tm.umax2(ud, ux);
+    tm.umax2(ud, ux, sc.keys + (it & 1) * WPC);
     if (WPC == 1) __syncwarp();
     const float hd = __uint_as_float(ud), hx = __uint_as_float(ux);
     if (!(hd < 1e38f) || !(hx < 1e38f)) return false;
