@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -698,6 +699,19 @@ void relocate(DevMech& dm, void* base) {
   dm.nasa_tmid = reloc(dm.nasa_tmid, base);
 }
 
+// Dynamic shared memory of at least bytes for launches of kernel f on the
+// current device. The limit belongs to the function, which the contexts of a
+// device have in common (and their creation may run in several threads): it is
+// only raised, so a smaller context does not refuse a larger one's launches.
+cudaError_t allow_shared(const void* f, int bytes) {
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
+  cudaFuncAttributes at;
+  const cudaError_t e = cudaFuncGetAttributes(&at, f);
+  if (e != cudaSuccess || at.maxDynamicSharedSizeBytes >= bytes) return e;
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 int configure_launch(dlbchem_ctx* c) {
   cudaDeviceProp prop;
   cudaError_t e = cudaGetDeviceProperties(&prop, c->device);
@@ -718,15 +732,14 @@ int configure_launch(dlbchem_ctx* c) {
   if (teams < 1) return fail(c, DLBCHEM_BAD_MECH, "mechanism too large: one cell's workspace exceeds shared memory");
   c->teams = teams;
   c->smem_bytes = int(team_bytes * teams) + 80 * 8;   // + the CTA's exp and nu tables
-  e = cudaFuncSetAttribute(dlb::rosenbrock_kernel_ptr(c->wpc, dlb::general_kernel(c->dm)), cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem_bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dlb::gate_kernel_ptr(c->wpc), cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem_bytes);
+  e = allow_shared(dlb::rosenbrock_kernel_ptr(c->wpc, dlb::general_kernel(c->dm)), c->smem_bytes);
+  if (e == cudaSuccess) e = allow_shared(dlb::gate_kernel_ptr(c->wpc), c->smem_bytes);
   c->rhs_L = make_rhs_layout(c->hm.nsp, c->hm.nrx, c->dm.N);
   c->rhs_teams = max_teams;
   while (c->rhs_teams > 1 && size_t(c->rhs_L.total) * 8 * c->rhs_teams + 640 > max_block) --c->rhs_teams;
   c->rhs_smem = c->rhs_L.total * 8 * c->rhs_teams + 80 * 8;
   const void* rhs = dlb::rhs_kernel_ptr(c->wpc, dlb::general_kernel(c->dm));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(rhs, cudaFuncAttributeMaxDynamicSharedMemorySize, c->rhs_smem);
+  if (e == cudaSuccess) e = allow_shared(rhs, c->rhs_smem);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->rhs_blocks, rhs, 32 * c->wpc * c->rhs_teams, c->rhs_smem);
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaFuncSetAttribute");
