@@ -98,11 +98,12 @@ typedef struct dlbchem_options {
                            warp of the team by an FP32 inverse of the iteration matrix and FP64
                            iterative refinement (residuals against the FP64 matrix) until the
                            last correction is below 2^-30 of the solution, at most 8 rounds;
-                           beyond that size, and for a step whose refinement does not converge,
-                           by the FP64 LU. 1: mixed precision: the refinement (beyond the size
-                           above with FP32 LU factors) stops when the estimated remaining error
-                           is below 1e-6 of the error weights, at most 3 rounds, the step redone
-                           with the FP64 LU if they do not converge. State, rates, error norm
+                           beyond that size, for a step whose refinement does not converge,
+                           and with atol below 1e-30 (corrections are floats), by the FP64
+                           LU. 1: mixed precision: the refinement (beyond the size above with
+                           FP32 LU factors) stops when the estimated remaining error is below
+                           1e-6 of the error weights, at most 3 rounds, the step redone with
+                           the FP64 LU if they do not converge. State, rates, error norm
                            and step control are FP64 in both. Fixed at create, which allocates
                            one matrix per resident team (SMs x CTAs per SM x teams; 22 MB at 54
                            unknowns on 152 SMs); if that fails, precision 0 runs the FP64 LU

@@ -117,6 +117,12 @@ struct IntegParams {
   int32_t precision, reserved;   // precision 1: FP32 LU + FP64 refinement
 };
 
+// Refined solves need an absolute tolerance of at least this: solutions, right-hand
+// sides and corrections pass through floats, whose normal range ends at 1.2e-38. A
+// correction is 2^-24 of the solution and has to be resolved where the solution is as
+// small as the tolerance, with two digits to spare for its weight.
+constexpr double kRefinedAtol = 1e-30;
+
 // One-warp teams keep the FP32 inverse of up to this many unknowns in shared memory.
 constexpr int kSharedX = 12;
 

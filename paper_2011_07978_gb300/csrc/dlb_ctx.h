@@ -59,10 +59,12 @@ struct dlbchem_ctx {
   // their slots (one per resident CTA)
   double* d_m64 = nullptr;
   unsigned* d_slots = nullptr;
+  // (none below kRefinedAtol: the FP64 LU takes every solve)
   void matrix_slots(dlb::KernelArgs& a) const {
-    a.m64 = d_m64;
+    const bool on = d_m64 && opt.atol >= dlb::kRefinedAtol;
+    a.m64 = on ? d_m64 : nullptr;
     a.slots = d_slots;
-    a.nslots = d_m64 ? num_sms * blocks_per_sm : 0;
+    a.nslots = on ? num_sms * blocks_per_sm : 0;
     a.slots_per_sm = blocks_per_sm;
   }
   int64_t ws_cap = 0;

@@ -1539,7 +1539,7 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
       float4* X4 = WPC == 1 && N <= kSharedX ? w.xs : reinterpret_cast<float4*>(w.g);
       if (inverse) {
         if (tm.tid < N)
-          w.inv_isc[tm.tid] = __frcp_rn(fmaf(float(P.rtol), fabsf(low_float(w.y0[tm.tid])), fmaxf(float(P.atol), 1e-30f)));
+          w.inv_isc[tm.tid] = __frcp_rn(fmaf(float(P.rtol), fabsf(low_float(w.y0[tm.tid])), fmaxf(float(P.atol), float(kRefinedAtol))));
         with_padded<WPC>(N, [&](auto np) { invert<WPC, decltype(np)::value>(tm, w.M, N, ld, w.inv, X4); });
       }
       // mixed: M goes, transposed, to the team's global copy, and its FP32
