@@ -1297,6 +1297,9 @@ __device__ __noinline__ void invert(const TeamThreads<WPC> tm, const double* M, 
 #pragma unroll
     for (int q = 0; q < NP / 4; ++q)
       put_x<NP>(X4 + q * N + row, make_float4(a[4 * q] * scale, a[4 * q + 1] * scale, a[4 * q + 2] * scale, a[4 * q + 3] * scale));
+    // a pivot above 2^126 has no normal reciprocal and got zero: its row of zeros
+    // would look converged, NaN takes the FP64 LU
+    if (scale == 0.f) put_x<NP>(X4 + row, make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f));
   }
   tm.sync();
 }

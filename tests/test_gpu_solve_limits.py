@@ -34,3 +34,17 @@ def test_traces_far_below_the_float_range_react(tmp_path, wpc, precision, atol, 
     g = run_gpu(dlb().Context(mech, team_warps=wpc, precision=precision, **opts), T, p, Y, 1e-7)
     assert_parity(g, o)
     assert np.all(np.abs(g[1][0] - o[1][0]) <= 1e-6 * o[1][0])
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("wpc", [1, 2, 4])
+def test_pivots_whose_reciprocal_is_no_normal_float(tmp_path, wpc, precision):
+    """1.5e-38 s in one step: the diagonal, 1/(gamma h) = 1.2e38, is a float and its reciprocal is
+    below 2^-126, where the hardware reciprocal gives zero."""
+    mech = decay(tmp_path, 1e36, hf=-1000.0)
+    T, p, Y = np.full(3, 1000.0), np.full(3, 1e5), np.array([[1.0, 0.5, 0.2], [0.0, 0.5, 0.8]])
+    opts = dict(rtol=1e-8, atol=1e-12)
+    o = oracle.Oracle(mech).integrate(T, p, Y, 1.5e-38, **opts)
+    assert abs(o[1][0, 0] / np.exp(-0.015) - 1.0) < 1e-7
+    ctx = dlb().Context(mech, team_warps=wpc, precision=precision, **opts)
+    assert_parity(run_gpu(ctx, T, p, Y, 1.5e-38), o)
