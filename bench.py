@@ -240,7 +240,7 @@ def time_form(dlbchem, mech_path, fstep, Td, pd, Yd, To, Yo, stream, *, schedule
     return {"cells_per_s": n / (ms / 1e3), "ms": ms, "integrator_ms": integ, "attempted_steps": total,
             "roofline_frac": ach / FP64_PEAK_TFLOPS, "achieved_tflops": ach, "integrated": st["integrated"],
             "mapped": st["mapped"], "failed": int((status < 0).sum().item()),
-            "fp64_fallbacks": st["fp64_fallbacks"] if precision else None}
+            "fp64_fallbacks": st["fp64_fallbacks"]}
 
 
 def mlp_forward_rate(dlbchem, dev, stream, n):

@@ -304,8 +304,11 @@ int dlbchem_nreactions(const dlbchem_ctx* ctx);
  *   surrogate), out[2] reference cell index with mapping 1 (-1 if none or
  *   with mapping 2; see dlbchem_last_mapping), out[3] team size in threads, out[4] teams per CTA,
  *   out[5] CTAs launched by the integrator, out[6] dynamic shared memory
- *   bytes per CTA, out[7] kernel launches in the call, out[8] steps whose
- *   mixed-precision refinement fell back to the FP64 LU, out[9] precision mode.
+ *   bytes per CTA, out[7] kernel launches in the call, out[8] steps
+ *   that took the FP64 LU where refined solves are the rule (up to 32 unknowns
+ *   per warp of the team, and all sizes in mixed precision): the refinement did
+ *   not converge, the cell had fallen back twice, or there is no matrix for it
+ *   (allocation at create, atol below 1e-30), out[9] precision mode.
  * Returns DLBCHEM_OK, BAD_ARG or CUDA.
  */
 int dlbchem_last_stats(dlbchem_ctx* ctx, int64_t out[10]);

@@ -1060,6 +1060,7 @@ int dlbchem_integrate(dlbchem_ctx* c, int64_t n, double dt, const double* T, con
   for (int i = 0; i < 10; ++i) c->stats[i] = 0;
   c->stats[2] = -1;
   c->stats[9] = c->opt.precision;
+  c->counted_last = false;
   if (n == 0) return DLBCHEM_OK;
   if (!T || !p || !Y || !T_out || !Y_out) return fail(c, DLBCHEM_BAD_ARG, "NULL array pointer");
   int rc = ensure_ws(c, n);
@@ -1130,16 +1131,16 @@ int dlbchem_integrate(dlbchem_ctx* c, int64_t n, double dt, const double* T, con
   a.P.max_steps = c->opt.max_steps; a.P.isothermal = c->opt.isothermal; a.P.precision = c->opt.precision;
   a.L = c->L;
   a.n = n; a.T = T; a.p = p; a.Y = Y; a.Tout = T_out; a.Yout = Y_out; a.steps = steps; a.status = status;
-  a.fallbacks = c->opt.precision == 1 ? c->d_counter + 2 : nullptr;   // counted for mixed precision only
+  a.fallbacks = c->counts_lu() ? c->d_counter + 2 : nullptr;
   c->matrix_slots(a);
-  if (c->opt.precision == 1 && (e = cudaMemsetAsync(c->d_counter + 2, 0, 8, s)) != cudaSuccess)
+  if (a.fallbacks && (e = cudaMemsetAsync(a.fallbacks, 0, 8, s)) != cudaSuccess)
     return cuda_fail(c, e, "cudaMemsetAsync");
   const bool listed = mapping || queue || surrogate || predictor;
   a.perm = listed ? c->w_list : nullptr;
   a.nqueue = listed ? c->w_total : nullptr;
   const int threads = 32 * c->wpc * c->teams;
   int64_t grid = (n + c->teams - 1) / c->teams;
-  if (queue || c->opt.precision == 1) {   // mixed precision indexes per-team scratch: persistent teams
+  if (queue || c->opt.precision == 1) {   // mixed precision: persistent teams
     e = cudaMemsetAsync(c->d_counter, 0, 8, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
     a.queue = 1; a.counter = c->d_counter; a.chunk = c->opt.chunk;
@@ -1158,6 +1159,7 @@ int dlbchem_integrate(dlbchem_ctx* c, int64_t n, double dt, const double* T, con
   rec(6);
   if (e != cudaSuccess) return cuda_fail(c, e, "mapping scatter");
   c->timed_last = timing;
+  c->counted_last = a.fallbacks != nullptr;
   c->last_n = n;
   c->last_mapping = mapping ? c->opt.mapping : (surrogate ? 3 : 0);
   c->last_listed = listed;
@@ -1251,7 +1253,7 @@ int dlbchem_last_stats(dlbchem_ctx* c, int64_t out[10]) {
     c->stats[1] = c->last_n - m;
     c->stats[2] = (c->last_mapping == 1 && int64_t(r) < c->last_n) ? int64_t(r) : -1;
   }
-  if (c->opt.precision == 1 && c->last_n > 0) {
+  if (c->counted_last) {
     unsigned long long fb = 0;
     if ((e = cudaMemcpy(&fb, c->d_counter + 2, 8, cudaMemcpyDeviceToHost)) != cudaSuccess) return cuda_fail(c, e, "cudaMemcpy");
     c->stats[8] = int64_t(fb);

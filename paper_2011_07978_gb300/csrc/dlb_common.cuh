@@ -265,7 +265,7 @@ struct KernelArgs {
   unsigned long long* counter;
   int chunk;
   int queue;
-  unsigned long long* fallbacks;   // steps whose FP32 refinement fell back to the FP64 LU
+  unsigned long long* fallbacks;   // steps that took the FP64 LU (null: not counted)
   // refined solves: per-team matrices (matrix_stride doubles each): a CTA takes
   // slot i of nslots (slots[i] 0 -> 1) for its teams while it runs
   double* m64;

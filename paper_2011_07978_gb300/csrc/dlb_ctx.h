@@ -67,6 +67,9 @@ struct dlbchem_ctx {
     a.nslots = on ? num_sms * blocks_per_sm : 0;
     a.slots_per_sm = blocks_per_sm;
   }
+  // where refined solves are the rule, the steps of a call that took the FP64 LU are counted
+  bool counts_lu() const { return opt.precision == 1 || dm.N <= 32 * wpc; }
+  bool counted_last = false;   // the last call did
   int64_t ws_cap = 0;
   uint8_t* w_flag = nullptr;
   double* w_ref_state = nullptr;

@@ -1565,7 +1565,10 @@ __device__ __forceinline__ void integrate_cell(const DevMech& m, const IntegPara
         else ok = lu_factor<WPC, float>(tm, w.M32, N, ld, w.invd32, w.perm32);
         if (!ok) { mixed = false; restore(); }
       }
-      if (!mixed && !inverse) ok = lu_factor<WPC, double>(tm, w.M, N, ld, w.invd, w.perm);
+      if (!mixed && !inverse) {
+        if (tm.tid == 0 && fallbacks) atomicAdd(fallbacks, 1ull);
+        ok = lu_factor<WPC, double>(tm, w.M, N, ld, w.invd, w.perm);
+      }
       for (int attempt = 0; attempt < 2; ++attempt) {
         bool conv = true;
         auto solve = [&](const double* b, double* x) {

@@ -125,11 +125,11 @@ extern "C" int dlbchem_integrate_static(dlbchem_ctx* c, int64_t n, double dt, co
   a.n = n; a.T = T; a.p = p; a.Y = Y; a.Tout = T_out; a.Yout = Y_out; a.steps = steps; a.status = status;
   a.perm = list; a.nqueue = total; a.queue = 1; a.counter = counter; a.chunk = c->opt.chunk;
   c->matrix_slots(a);   // allocated once, at creation
-  // mixed precision: count the steps whose refinement fell back to the FP64
-  // LU in the context's own counter (allocated at creation)
-  if (c->opt.precision == 1) {
+  // the steps that take the FP64 LU are counted in the context's own counter
+  // (allocated at creation)
+  if (c->counts_lu()) {
     a.fallbacks = c->d_counter + 2;
-    e = cudaMemsetAsync(c->d_counter + 2, 0, 8, s);
+    e = cudaMemsetAsync(a.fallbacks, 0, 8, s);
     if (e != cudaSuccess) return fail(c, DLBCHEM_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
   }
   int64_t grid = (n + c->teams - 1) / c->teams;
@@ -142,6 +142,7 @@ extern "C" int dlbchem_integrate_static(dlbchem_ctx* c, int64_t n, double dt, co
   c->last_mapping = 0;
   c->last_listed = 0;
   c->timed_last = false;
+  c->counted_last = a.fallbacks != nullptr;
   for (int i = 0; i < 10; ++i) c->stats[i] = 0;
   c->stats[0] = n; c->stats[2] = -1; c->stats[3] = 32 * c->wpc; c->stats[4] = c->teams;
   c->stats[5] = grid; c->stats[6] = c->smem_bytes; c->stats[7] = 1 + (steps ? 12 : 0) + 1;
