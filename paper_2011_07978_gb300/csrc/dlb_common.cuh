@@ -123,7 +123,10 @@ struct IntegParams {
 // small as the tolerance, with two digits to spare for its weight.
 constexpr double kRefinedAtol = 1e-30;
 
-// One-warp teams keep the FP32 inverse of up to this many unknowns in shared memory.
+// One-warp teams keep the FP32 inverse of up to this many unknowns in shared memory
+// (10-species steps: 84 kcycles, 87 with the inverse in L2). The next padded size, 20,
+// needs a larger workspace: the inverse has to end before D (see make_layout), and from
+// 14 unknowns on it would not.
 constexpr int kSharedX = 12;
 
 // Offsets (in doubles) of one team's workspace inside dynamic shared memory.
@@ -160,9 +163,11 @@ __host__ inline WsLayout make_layout(int nsp, int nrx, int CH, int N, int ld, in
   L.scal = take(48);
   L.perm = take((N + 1) / 2 + 1);
   L.M32 = L.invd32 = L.perm32 = L.rr = L.dx = L.isc = 0;
-  // refined solves: weights and right-hand side over the Jacobian-only arrays
-  // dwdT .. dlt (dead from the assembly of one step to the next), published
-  // rows (dead during the rate evaluations too) behind them up to scal
+  // refined solves: weights, right-hand side, first solution and a shared inverse
+  // over the Jacobian-only arrays dwdT .. dlt (dead from the assembly of one step
+  // to the next). They live across the rate evaluations of stages 2 and 3, which
+  // write D, so they end before it; what only the inversion uses (reciprocals,
+  // published rows) may lie over D too, up to scal. Without room all are appended.
   L.w32 = L.v = L.xf = L.xs = L.invs = L.rows = 0;
   if (N <= CH) {
     auto vectors = [&](auto&& take2) {
@@ -175,7 +180,7 @@ __host__ inline WsLayout make_layout(int nsp, int nrx, int CH, int N, int ld, in
     };
     int o2 = L.dwdT;
     vectors([&](int n) { int r = o2; o2 += (n + 1) & ~1; return r; });
-    if (o2 > L.scal) vectors(take);
+    if (L.invs > L.D || o2 > L.scal) vectors(take);
   } else if (mixed) {
     // FP32 factors over the first half of M (the FP64 matrix is kept in a
     // global per-team scratch); pivots and refinement vectors over the
