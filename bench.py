@@ -46,27 +46,49 @@ METRIC = "chemistry cells/s per dt at stated T/Y error vs FP64 oracle; frac of F
 # FMA lanes per clock per SM x 2 flop (= the 1.25 TFLOP/s nominal figure).
 FP64_PEAK_TFLOPS = 152 * 2.07e9 * 2 * 2 / 1e12
 # dram__bytes_read.sum + dram__bytes_write.sum of one FP64 integrator launch
-# (rosenbrock_kernel<2, false>) from ncu per integrated cell (4,040,960 B
-# read, 0 written, 912 cells integrated on the 8,192-cell bimodal field with
+# (rosenbrock_kernel<2, false>) from ncu per integrated cell (4.41 MB read and
+# 0.11 MB written, 912 cells integrated on the 8,192-cell bimodal field with
 # bucket mapping), scaled by the cells the benchmark's launch integrates; None
-# whenever the kernel has changed since the capture.
+# whenever the kernel's memory accesses have changed since the capture.
 INTEGRATOR_TRAFFIC_BYTES_PER_CELL = 4520960 / 912
 N_F = 3   # function evaluations per Rosenbrock step (stage 4 reuses stage 3's)
+FP32_PEAK_TFLOPS = 152 * 2.07e9 * 128 * 2 / 1e12   # 128 FP32 FMA lanes per clock per SM
 PAPER_CONTEXT = ("paper (DLBFoam, arXiv 2011.07978): load balancing + reference mapping speed the CPU "
                  "chemistry step up by about 10x (Spray A, 256 MPI ranks on 2x64-core AMD EPYC Rome nodes, "
                  "FP64; chi_su 9.87 LB+RM, 2.57 LB only); context, not a target")
 
 
 def flops_per_step(m) -> float:
-    """Algorithmic FP64 flops of one attempted step of the 4-stage Rosenbrock
-    method: (2/3) N^3 for the LU of the iteration matrix, 8 N^2 for its four
+    """Flops of one attempted step of the 4-stage Rosenbrock method with direct
+    FP64 solves: (2/3) N^3 for the LU of the iteration matrix, 8 N^2 for its four
     pairs of triangular solves, n_f (25 R + 15 N_sp) for the n_f = 3 rate and
     right-hand-side evaluations, 90 R + 3 N^2 for the analytic Jacobian and
     the assembly of the iteration matrix. exp and log are not flops here;
-    transcendentals_per_step counts them."""
+    transcendentals_per_step counts them. The measure of the same result by
+    another solver; what the integrator executes is step_work's."""
     nsp, nrx = m.nsp, m.nrx
     N = nsp + 1
     return (2.0 / 3.0) * N**3 + 8.0 * N**2 + N_F * (25 * nrx + 15 * nsp) + 90 * nrx + 3 * N**2
+
+
+def step_work(m, precision=0, team_warps=0) -> dict:
+    """Flops of one attempted step as the integrator does it, by the unit that
+    executes them. Rates, Jacobian and assembly are FP64. Up to 32 unknowns per
+    warp of the team (128 with the automatic teams) the solves are an FP32 inverse (2 N^3) and per solve
+    2 N^2 for each product with it (three, two in mixed precision: the first
+    solution and its corrections) and each residual before a correction: FP64,
+    but the first of two above 32 unknowns, which is in paired floats (counted as
+    2 N^2 there). Beyond that size the LU, FP64 or in mixed precision FP32 with
+    one FP64 residual."""
+    nsp, nrx = m.nsp, m.nrx
+    N = nsp + 1
+    f64 = float(N_F * (25 * nrx + 15 * nsp) + 90 * nrx + 3 * N**2)
+    lu = (2.0 / 3.0) * N**3 + 8.0 * N**2
+    if N > 32 * (team_warps or (1 if N <= 32 else 2 if N <= 64 else 4)):
+        return {"f64": f64 + (8.0 * N**2 if precision else lu), "f32": lu + 8.0 * N**2 if precision else 0.0}
+    products, residuals = (2, 1) if precision else (3, 2)
+    paired = 1 if residuals == 2 and N > 32 else 0
+    return {"f64": f64 + 8.0 * N**2 * (residuals - paired), "f32": 2.0 * N**3 + 8.0 * N**2 * (products + paired)}
 
 
 def transcendentals_per_step(m) -> dict:
@@ -215,7 +237,7 @@ def conservation(mech, T, Y, To, Yo):
             "element_defect_max_rel": float(rel.max()) if rel.numel() else 0.0}
 
 
-def time_form(dlbchem, mech_path, fstep, Td, pd, Yd, To, Yo, stream, *, schedule, mapping, precision, warm=1):
+def time_form(dlbchem, mech_path, mech, Td, pd, Yd, To, Yo, stream, *, schedule, mapping, precision, warm=1):
     """One comparison form on the full field: warm-up calls (the first gives
     the queue's cost keys), then one call timed with CUDA events."""
     import torch
@@ -236,7 +258,7 @@ def time_form(dlbchem, mech_path, fstep, Td, pd, Yd, To, Yo, stream, *, schedule
     integ = ctx.last_timing()["integrator_ms"]
     st = ctx.last_stats()
     total = int(steps.sum().item())
-    ach = fstep * total / (integ / 1e3) / 1e12
+    ach = step_work(mech, precision)["f64"] * total / (integ / 1e3) / 1e12
     return {"cells_per_s": n / (ms / 1e3), "ms": ms, "integrator_ms": integ, "attempted_steps": total,
             "roofline_frac": ach / FP64_PEAK_TFLOPS, "achieved_tflops": ach, "integrated": st["integrated"],
             "mapped": st["mapped"], "failed": int((status < 0).sum().item()),
@@ -328,7 +350,7 @@ def main():
     ap.add_argument("--team-warps", type=int, default=0, choices=[0, 1, 2, 4],
                     help="warps per cell (0 = the library's automatic choice)")
     ap.add_argument("--precision", default="fp64", choices=["fp64", "mixed"],
-                    help="mixed: FP32 LU of the iteration matrix with FP64 refinement")
+                    help="mixed: linear solves refined to 1e-6 of the error weights only")
     ap.add_argument("--mlp-only", type=int, default=0, metavar="CELLS",
                     help="only time the network's forward pass on CELLS rows and print its JSON")
     args = ap.parse_args()
@@ -403,11 +425,11 @@ def main():
     ms_per_step = dev_ms / args.steps
     value = job_throughput(n, world, ms_per_step)
 
-    # roofline of the integrator kernel (algorithmic flops / its event-timed duration)
-    fstep = flops_per_step(mech)
-    flops_launch = fstep * total_steps / args.steps
+    # roofline of the integrator kernel (the flops of each unit / its event-timed duration)
+    fstep = step_work(mech, prec, args.team_warps)
     integ_avg_ms = float(np.mean(integ_ms))
-    achieved = flops_launch / (integ_avg_ms / 1e3) / 1e12
+    rate = lambda flops: flops * total_steps / args.steps / (integ_avg_ms / 1e3) / 1e12
+    achieved, achieved32 = rate(fstep["f64"]), rate(fstep["f32"])
     stats = ctx.last_stats()
     status_h = status.cpu().numpy()
     cons = conservation(mech, Td, Yd, To, Yo)
@@ -436,7 +458,7 @@ def main():
     line = {
         "metric": METRIC, "value": value, "unit": "cells/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "f64" if args.precision == "fp64" else "f64 (LU in f32, f64 refinement)",
+        "vs_baseline": None, "dtype": "f64" if args.precision == "fp64" else "f64 (solves by an f32 inverse, f64 refinement)",
         "data": "synthetic",
         "config": {"workload": f"bimodal {n} cells, 53 species / 325 reactions (seeded synthetic), p 20 bar, "
                                f"dt 1e-5 s, rtol 1e-5, atol 1e-8, {'FP64' if args.precision == 'fp64' else 'mixed precision'}",
@@ -449,8 +471,15 @@ def main():
                                  if args.precision == "fp64" and INTEGRATOR_TRAFFIC_BYTES_PER_CELL else None),
                      "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum per integrated cell, "
                                        "8,192-cell capture, scaled by the cells integrated per launch",
-                     "kernel": "rosenbrock_kernel", "flops_per_step": fstep,
-                     "flops_formula": "(2/3)N^3 + 8N^2 + 3(25R + 15Nsp) + 90R + 3N^2, N = Nsp + 1",
+                     "kernel": "rosenbrock_kernel", "flops_per_step": fstep["f64"],
+                     "flops_formula": "FP64 work: 3(25R + 15Nsp) + 90R + 3N^2 + 8N^2 (residuals), N = Nsp + 1",
+                     "fp32": {"flops_per_step": fstep["f32"], "achieved": achieved32, "peak": FP32_PEAK_TFLOPS,
+                              "frac": achieved32 / FP32_PEAK_TFLOPS,
+                              "work": "inverse and its products, first residual, beside the FP64 unit"},
+                     "lu_equivalent": {"flops_per_step": flops_per_step(mech), "rate": rate(flops_per_step(mech)),
+                                       "unit": "TFLOP/s",
+                                       "note": "the same steps counted with an FP64 LU and triangular solves, "
+                                               "which do not run here: no fraction of a peak"},
                      "transcendentals_per_step": transcendentals_per_step(mech),
                      "steps_per_launch": total_steps / args.steps, "launch_ms": integ_avg_ms,
                      "peak_source": "derived: 152 SMs x 2.07 GHz x 2 FP64 FMA/clk/SM x 2",
@@ -480,7 +509,7 @@ def main():
             same = (kw["schedule"] == sched and kw["mapping"] == args.mapping and kw["precision"] == prec)
             if same or (kw["mapping"] == 2 and HEADLINE_MAPPING != 2):
                 continue
-            arms[name] = time_form(dlbchem, mech_path, fstep, Td, pd, Yd, scratch_T, scratch_Y, stream, **kw)
+            arms[name] = time_form(dlbchem, mech_path, mech, Td, pd, Yd, scratch_T, scratch_Y, stream, **kw)
         line["forms"] = arms
     if rank == 0 and not args.no_cpu_baseline:
         import oracle
