@@ -114,7 +114,7 @@ __host__ __device__ inline bool general_kernel(const DevMech& m) { return m.nplo
 struct IntegParams {
   double rtol, atol, hmin_frac, dt;
   int32_t max_steps, isothermal;
-  int32_t precision, reserved;   // precision 1: FP32 LU + FP64 refinement
+  int32_t precision, reserved;   // precision 1: solves refined to 1e-6 of the error weights
 };
 
 // Refined solves need an absolute tolerance of at least this: solutions, right-hand

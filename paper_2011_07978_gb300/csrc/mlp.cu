@@ -4,8 +4,9 @@
 // cores (tcgen05.mma, kind::f16) in BF16 with the FP32 accumulator in tensor
 // memory: inference as one whole-network kernel per 128-row tile, training
 // layer by layer (FP32 master weights and activations are rounded to BF16
-// when a tile is staged in shared memory); the MSE gradient, bias gradients
-// and Adam are FP32 element kernels.
+// when a tile is staged in shared memory), the loss, its gradient and SiLU' in
+// the epilogues, the bias sums beside the staging of the weight gradients, all
+// in FP32. Adam is an FP32 element kernel.
 //
 // Inputs of the network for one cell: x = [T/1000, ln p, Y_1..Y_nsp, ln dt];
 // outputs: [ln(attempted steps), dT, dY_1..dY_nsp]. Both are normalised by
